@@ -33,7 +33,7 @@ KERNEL_SOURCES = {
     "ray_step": ["ray_kernels.cu", "mesh_kernels.h"],
     "kick_drift": ["mesh_kernels.cu"],
     "cic_scatter": ["mesh_kernels.cu"],
-    "kspace": ["mesh_kernels.cu", "xpass_kernels.cu", "tma.h"],
+    "kspace": ["mesh_kernels.cu", "fft_passes.cu", "tma.h"],
 }
 
 
@@ -200,14 +200,21 @@ def algorithmic_bytes(W):
     rays = W.n_rays
     return {
         "cic_scatter": 3 * 4 * npart + mesh,                 # positions read + density written
-        # density spectrum read + 3 gradient spectra written; on the split path (mesh sides 256, 512, 1024) the
-        # x-pass also zeroes the consumed density for the next deposit
-        "kspace": spec + 3 * spec + (mesh if W.n_mesh in (256, 512, 1024) else 0),
+        # density spectrum read; 3 gradient spectra written, on the split path (own FFT passes) 2: the x component
+        # and the one that both d_y and d_z are taken from
+        "kspace": spec + (2 if own_fft(W) else 3) * spec,
         "kick_drift": 4 * mesh + 2 * 2 * 3 * 4 * npart,      # 3 fields read, density written, disp/mom r+w
         "ray_step": 2 * rays * (16 + 8 + 16 + 16),           # ray state read and written (slab reads extra)
-        "fft_r2c": mesh + spec,
-        "fft_c2r": 3 * (spec + mesh),
+        # own passes: z (density read and zeroed, spectrum written) and y (read, written)
+        "fft_r2c": 2 * mesh + 3 * spec if own_fft(W) else mesh + spec,
+        # own passes: y (2 spectra read, 3 written) and z (3 read, 3 fields written)
+        "fft_c2r": 8 * spec + 3 * mesh if own_fft(W) else 3 * (spec + mesh),
     }
+
+
+def own_fft(W):
+    """Whether the library's own FFT passes run the Poisson solve of this mesh (else cuFFT and the k-space kernel)."""
+    return W.n_mesh in (256, 512, 1024)
 
 
 # ----------------------------------------------------------------------------------------------- GPU arm
@@ -259,6 +266,8 @@ def run_gpu(args, W, world, rank, local):
         ctx.hrt_set_ray_mesh(raymesh_config(hrt, W))
         ray_launches = 5
 
+    # own kernels per Poisson solve: the FFT passes along z, y, x and back, or the k-space kernel between cuFFT plans
+    solve_launches = 5 if own_fft(W) else 1
     # the context sorts particles given by the caller before their first force, then every sort_every particle
     # steps (6 own launches: cell keys, three scan passes, inversion, gather)
     sort_every = 8 if args.sort_every is None else args.sort_every
@@ -278,11 +287,11 @@ def run_gpu(args, W, world, rank, local):
         for _ in range(k):
             if pos == len(grid) - 1:
                 reset()
-                launches += 3 + (6 if sort_every > 0 else 0)  # sort, CIC scatter, k-space pass, ray initialisation
+                launches += 2 + solve_launches + (6 if sort_every > 0 else 0)  # sort, CIC scatter, solve, ray initialisation
                 pos = 0
             n = pos + 1
             ctx.hrt_step(grid[n], slots.get(n, -1))
-            launches += 2 + ray_launches  # ray step, kick-drift-deposit, k-space pass (x-pass on the split path)
+            launches += 1 + solve_launches + ray_launches  # kick-drift-deposit, Poisson solve, ray step
             since_sort[0] += 1
             if sort_every > 0 and since_sort[0] >= sort_every:
                 launches += 6

@@ -171,11 +171,11 @@ hrt_status hrt_pm_destroy(hrt_pm* pm); /* NULL is fine; synchronises the stream 
  * k-space kernel.  Returns HRT_ERR_CUDA if cuFFT refuses the callback. */
 hrt_status hrt_pm_set_fused(hrt_pm* pm, int32_t on);
 
-/* Split path of hrt_pm_solve (on by default for n = 256, 512, 1024): batched 2D (y, z) cuFFT plans over the
- * x-planes and one x-pass kernel between them that does the forward FFT along x, the k-space step of
- * hrt_kspace_gradient and the inverse FFTs along x, so that no 3D spectrum is written or read twice.  Same
- * results as the 3D path (FP32 rounding of a different FFT order).  on = 0 returns to 3D cuFFT plans and the
- * separate k-space kernel.  HRT_ERR_INVALID_ARG for other mesh sides. */
+/* Split path of hrt_pm_solve (on by default for n = 256, 512, 1024): the library's own FFT passes along z, y and x,
+ * with the k-space step of hrt_kspace_gradient inside the x pass, and back along y and z, so that every spectrum
+ * crosses memory once per axis and no 3D spectrum is formed.  Same results as the 3D path (FP32 rounding of a
+ * different FFT order).  on = 0 returns to 3D cuFFT plans and the separate k-space kernel.  HRT_ERR_INVALID_ARG for
+ * other mesh sides. */
 hrt_status hrt_pm_set_split(hrt_pm* pm, int32_t on);
 
 /* grad[3][n^3] <- gradient of phi from rho[n^3] (rho is overwritten as FFT scratch);

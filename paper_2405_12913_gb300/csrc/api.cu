@@ -19,11 +19,11 @@
 #include "common.h"
 #include "context.h"
 #include "cosmo.h"
+#include "fft_passes.h"
 #include "kspace_callback.h"
 #include "mesh_kernels.h"
 #include "mlp.h"
 #include "raymesh.h"
-#include "xpass.h"
 
 extern "C" const unsigned char hrt_kspace_callback_fatbin[];
 extern "C" const size_t hrt_kspace_callback_fatbin_size;
@@ -301,23 +301,24 @@ struct hrt_pm {
   bool have_cb3 = false, have_cb2 = false;
   hrt::KspaceCallbackInfo* cb_info = nullptr;  // device: [0] particle fields, [1] ray fields
   size_t work_bytes = 0;
-  // split path (the default where supported): batched 2D (y, z) plans over the x-planes, and the
-  // x-pass kernel between them (forward x-FFT, k-space step, inverse x-FFTs)
-  bool split = false;
-  cufftHandle r2c2d = 0, c2r2d = 0;
-  bool have_r2c2d = false, have_c2r2d = false;
-  float2* xtw = nullptr;    // x-FFT twiddles
-  int* xerr = nullptr;      // device error word of the kernels that wait for TMA copies (x-pass, tiled deposit)
-  bool last_split = false;  // rho_hat holds the (y, z)-transformed density of the split path
+  // split path (the default where supported): the library's own FFT passes along z, y and x (fft_passes.h).  Their
+  // spectra lie in rho_hat, grad_hat and split_hat (1, or 3 with ray fields).
+  bool split = false, have_split = false;
+  hrt::FftPlan fft;
+  float2* twiddles = nullptr;
+  void* split_hat = nullptr;
+  int* xerr = nullptr;      // device error word of the kernels that wait for TMA copies (FFT passes, tiled deposit)
+  bool last_split = false;  // the last solve took the split path, which leaves no 3D spectrum in rho_hat
 };
 
 namespace hrt {
 
 static size_t spectrum_bytes(int64_t n) { return static_cast<size_t>(n) * n * (n / 2 + 1) * sizeof(float2); }
-// Bytes of one spectrum buffer: the half spectrum, or the padded split layout where the split path exists.
-static size_t spectrum_alloc(int64_t n) {
-  return xpass_supported(n) ? static_cast<size_t>(n) * n * xpass_row(n) * sizeof(float2) : spectrum_bytes(n);
-}
+// Bytes of one spectrum buffer: the half spectrum, or the padded layout of the FFT passes where they exist.
+static size_t spectrum_alloc(int64_t n) { return fft_supported(n) ? fft_spectrum_bytes(n) : spectrum_bytes(n); }
+// Spectra the FFT passes need beyond the 4 (6 with ray fields) of the 3D path: the transformed density, two spectra
+// per filter set out of the x-pass and all fields but the first between the inverse passes.
+static int split_spectra(int32_t n_ray) { return n_ray > 0 ? 3 : 1; }
 
 static bool fusable(int64_t n) { return n >= 8 && n <= 1024 && (n & (n - 1)) == 0; }
 
@@ -348,36 +349,30 @@ static void pm_set_work(hrt_pm* pm) {
     cufftSetWorkArea(pm->c2r_cb2, pm->work);
     cufftSetStream(pm->c2r_cb2, pm->stream);
   }
-  for (int i = 0; i < 2; ++i) {
-    if (!(i == 0 ? pm->have_r2c2d : pm->have_c2r2d)) continue;
-    cufftHandle p = i == 0 ? pm->r2c2d : pm->c2r2d;
-    cufftSetWorkArea(p, pm->work);
-    cufftSetStream(p, pm->stream);
-  }
 }
 
-// Batched 2D (y, z) plans over the n x-planes, spectra rows padded to xpass_row(n), and the x-FFT twiddles.
-static hrt_status pm_make_split(hrt_pm* pm, size_t* work) {
-  const long long n = pm->n, nzp = xpass_row(pm->n);
-  long long dims[2] = {n, n}, real_embed[2] = {n, n}, spec_embed[2] = {n, nzp};
-  size_t w1 = 0, w2 = 0;
-  HRT_CUFFT(cufftCreate(&pm->r2c2d));
-  pm->have_r2c2d = true;
-  HRT_CUFFT(cufftSetAutoAllocation(pm->r2c2d, 0));
-  HRT_CUFFT(cufftMakePlanMany64(pm->r2c2d, 2, dims, real_embed, 1, n * n, spec_embed, 1, n * nzp, CUFFT_R2C, n, &w1));
-  HRT_CUFFT(cufftCreate(&pm->c2r2d));
-  pm->have_c2r2d = true;
-  HRT_CUFFT(cufftSetAutoAllocation(pm->c2r2d, 0));
-  HRT_CUFFT(cufftMakePlanMany64(pm->c2r2d, 2, dims, spec_embed, 1, n * nzp, real_embed, 1, n * n, CUFFT_C2R, n, &w2));
-  *work = std::max(w1, w2);
+// Buffers, twiddles and tensor maps of the FFT passes.
+static hrt_status pm_make_split(hrt_pm* pm) {
+  const size_t sp = spectrum_alloc(pm->n);
+  HRT_TRY(device_alloc(&pm->split_hat, sp * split_spectra(pm->n_ray), pm->stream, "spectra of the FFT passes"));
   std::vector<float2> tw;
-  xpass_twiddles(pm->n, tw);
-  HRT_TRY(device_alloc(reinterpret_cast<void**>(&pm->xerr), sizeof(int), pm->stream, "x-pass error word"));
+  fft_twiddles(pm->n, tw);
+  HRT_TRY(device_alloc(reinterpret_cast<void**>(&pm->xerr), sizeof(int), pm->stream, "FFT pass error word"));
   HRT_CUDA(cudaMemsetAsync(pm->xerr, 0, sizeof(int), pm->stream));
-  HRT_TRY(device_alloc(reinterpret_cast<void**>(&pm->xtw), tw.size() * sizeof(float2), pm->stream, "twiddles"));
-  HRT_CUDA(cudaMemcpyAsync(pm->xtw, tw.data(), tw.size() * sizeof(float2), cudaMemcpyHostToDevice, pm->stream));
+  HRT_TRY(device_alloc(reinterpret_cast<void**>(&pm->twiddles), tw.size() * sizeof(float2), pm->stream, "twiddles"));
+  HRT_CUDA(cudaMemcpyAsync(pm->twiddles, tw.data(), tw.size() * sizeof(float2), cudaMemcpyHostToDevice, pm->stream));
   // the host vector must outlive the copy
   HRT_CUDA(cudaStreamSynchronize(pm->stream));
+  const int n_mid = pm->n_ray > 0 ? 4 : 2, fields = 3 + pm->n_ray;
+  void *mid[4], *rest[kFftMaxFields - 1];
+  char* pool[2] = {static_cast<char*>(pm->grad_hat), static_cast<char*>(pm->split_hat)};
+  for (int i = 0; i < n_mid; ++i) mid[i] = pool[0] + i * sp;
+  for (int i = 1; i < fields; ++i) {
+    const int k = n_mid + i - 1;
+    rest[i - 1] = k < fields ? pool[0] + k * sp : pool[1] + (k - fields) * sp;
+  }
+  HRT_TRY(fft_plan(pm->fft, pm->n, fields, pm->rho_hat, mid, rest, pm->twiddles, pm->xerr));
+  pm->have_split = pm->split = true;
   return HRT_OK;
 }
 
@@ -397,16 +392,11 @@ static hrt_status pm_make(int64_t n, double box, int32_t n_ray, cudaStream_t s, 
   HRT_CUFFT(cufftSetAutoAllocation(pm->c2r, 0));
   HRT_CUFFT(cufftMakePlanMany64(pm->c2r, 3, dims, nullptr, 1, 0, nullptr, 1, 0, CUFFT_C2R, 1, &w2));
   pm->work_bytes = std::max(w1, w2);
-  if (xpass_supported(n)) {
-    size_t w3 = 0;
-    HRT_TRY(pm_make_split(pm, &w3));
-    pm->work_bytes = std::max(pm->work_bytes, w3);
-    pm->split = true;
-  }
   HRT_TRY(device_alloc(&pm->work, pm->work_bytes, s, "cuFFT work area"));
   pm_set_work(pm);
   HRT_TRY(device_alloc(&pm->rho_hat, spectrum_alloc(n), s, "rho_hat"));
   HRT_TRY(device_alloc(&pm->grad_hat, spectrum_alloc(n) * (3 + n_ray), s, "gradient spectra"));
+  if (fft_supported(n)) HRT_TRY(pm_make_split(pm));
   return HRT_OK;
 }
 
@@ -447,9 +437,8 @@ static void pm_release(hrt_pm* pm) {
   if (pm->have_c2r) cufftDestroy(pm->c2r);
   if (pm->have_cb3) cufftDestroy(pm->c2r_cb3);
   if (pm->have_cb2) cufftDestroy(pm->c2r_cb2);
-  if (pm->have_r2c2d) cufftDestroy(pm->r2c2d);
-  if (pm->have_c2r2d) cufftDestroy(pm->c2r2d);
-  device_free(pm->xtw, pm->stream);
+  device_free(pm->twiddles, pm->stream);
+  device_free(pm->split_hat, pm->stream);
   device_free(pm->xerr, pm->stream);
   device_free(pm->work, pm->stream);
   device_free(pm->rho_hat, pm->stream);
@@ -498,8 +487,8 @@ static KspaceCallbackInfo callback_info(const hrt_pm* pm, const float* tab, cons
 }
 
 // before_fields (optional): an event the stream waits for before the C2Rs overwrite grad / ray_grad (work on
-// another stream that still reads the previous fields).  clear_rho: on the split path the x-pass sets rho to
-// zero once the 2D R2C has consumed it (*cleared tells whether it did), which spares the next deposit its memset.
+// another stream that still reads the previous fields).  cleared: on the split path the forward z-pass sets rho to
+// zero once it has read it (*cleared tells whether it did), which spares the next deposit its memset.
 static hrt_status pm_solve(hrt_pm* pm, float* rho, double pref, const hrt_filter* f, float* grad,
                            const hrt_filter* fr, float* ray_grad, hrt_ctx* prof = nullptr,
                            cudaEvent_t before_fields = nullptr, bool* cleared = nullptr) {
@@ -513,41 +502,24 @@ static hrt_status pm_solve(hrt_pm* pm, float* rho, double pref, const hrt_filter
   if (rays) HRT_TRY(pm_tables(pm, *fr, &pm->tab_b, &pm->key_b));
   pm->last_split = pm->split && !pm->fused;
   if (pm->last_split) {
-    const int64_t n = pm->n;
-    const size_t sp = spectrum_alloc(n);
-    char* gh = static_cast<char*>(pm->grad_hat);
     {
       PhaseScope ps(pc, 3);
-      HRT_CUFFT(cufftExecR2C(pm->r2c2d, rho, static_cast<cufftComplex*>(pm->rho_hat)));
-    }
-    auto set = [&](const float* tab, const hrt_filter& flt, int n_out, char* out) {
-      XpassSet x{};
-      x.wxy = tab;
-      x.wz = tab + n;
-      x.g = flt.g_table;
-      x.g_nk = flt.g_nk;
-      x.g_inv_dk = flt.g_table ? static_cast<float>((flt.g_nk - 1) / flt.g_kmax) : 0.f;
-      x.n_out = n_out;
-      x.out = reinterpret_cast<float2*>(out);
-      return x;
-    };
-    const XpassSet xa = set(pm->tab_a, *f, 3, gh);
-    const XpassSet xb = rays ? set(pm->tab_b, *fr, pm->n_ray, gh + 3 * sp) : XpassSet{};
-    {
-      PhaseScope ps(pc, 4);
-      HRT_TRY(launch_xpass(pm->rho_hat, n, pm->box, pref, pm->xtw, xa, xb, pm->xerr, pm->stream,
-                           cleared ? rho : nullptr, cleared ? n * n * n : 0));
+      HRT_TRY(launch_fft_forward(pm->fft, rho, cleared != nullptr, pm->stream));
       if (cleared) *cleared = true;
     }
-    if (before_fields) HRT_CUDA(cudaStreamWaitEvent(pm->stream, before_fields, 0));
+    auto set = [&](const float* tab, const hrt_filter& flt) {
+      return FftSet{tab, tab + pm->n, flt.g_table, flt.g_nk,
+                    flt.g_table ? static_cast<float>((flt.g_nk - 1) / flt.g_kmax) : 0.f};
+    };
+    {
+      PhaseScope ps(pc, 4);
+      const FftSet a = set(pm->tab_a, *f), b = rays ? set(pm->tab_b, *fr) : FftSet{};
+      HRT_TRY(launch_fft_x(pm->fft, pm->box, pref, a, rays ? &b : nullptr, pm->stream));
+    }
     PhaseScope ps(pc, 5);
-    const size_t mb = static_cast<size_t>(n) * n * n;
-    for (int j = 0; j < 3; ++j)
-      HRT_CUFFT(cufftExecC2R(pm->c2r2d, reinterpret_cast<cufftComplex*>(gh + j * sp), grad + j * mb));
-    if (rays)
-      for (int j = 0; j < pm->n_ray; ++j)
-        HRT_CUFFT(cufftExecC2R(pm->c2r2d, reinterpret_cast<cufftComplex*>(gh + (3 + j) * sp), ray_grad + j * mb));
-    return HRT_OK;
+    HRT_TRY(launch_fft_inverse_y(pm->fft, pm->box, rays, pm->stream));
+    if (before_fields) HRT_CUDA(cudaStreamWaitEvent(pm->stream, before_fields, 0));
+    return launch_fft_inverse_z(pm->fft, grad, rays ? ray_grad : nullptr, pm->stream);
   }
   {
     PhaseScope ps(pc, 3);
@@ -600,7 +572,7 @@ static hrt_status ctx_mark(hrt_ctx* ctx, hrt_status s) {
 
 // The opt-in check for NaN and infinity: scans the given arrays on the context's stream (after everything queued
 // so far), waits within the host wait limit and returns HRT_ERR_NONFINITE if any value is not finite.  Also
-// reports a kernel that gave up waiting for its own copies (the x-pass error word) as HRT_ERR_TIMEOUT.
+// reports a kernel that gave up waiting for its own copies (the FFT passes' error word) as HRT_ERR_TIMEOUT.
 struct ScanItem {
   const void* p;
   int64_t n;
@@ -994,7 +966,7 @@ hrt_status hrt_pm_set_fused(hrt_pm* pm, int32_t on) {
 
 hrt_status hrt_pm_set_split(hrt_pm* pm, int32_t on) {
   if (!pm) return fail(HRT_ERR_INVALID_ARG, "pm is NULL");
-  if (on && !pm->have_r2c2d) return fail(HRT_ERR_INVALID_ARG, "the split path needs a mesh side of 256, 512 or 1024");
+  if (on && !pm->have_split) return fail(HRT_ERR_INVALID_ARG, "the split path needs a mesh side of 256, 512 or 1024");
   pm->split = on != 0;
   return HRT_OK;
 }
@@ -1608,6 +1580,7 @@ hrt_status hrt_workspace_bytes(const hrt_config* cfg, int64_t n_rays, size_t* by
   const size_t n = cfg->n_mesh, mesh = n * n * n * sizeof(float), np = cfg->n_side * cfg->n_side * cfg->n_side;
   size_t b = 6 * np * sizeof(float) + mesh * (4 + cfg->ray_fields);
   b += spectrum_alloc(cfg->n_mesh) * (1 + 3 + cfg->ray_fields) + 2 * spectrum_bytes(cfg->n_mesh);  // + cuFFT work
+  if (fft_supported(cfg->n_mesh)) b += fft_spectrum_bytes(cfg->n_mesh) * split_spectra(cfg->ray_fields);
   b += static_cast<size_t>(n_rays) * (2 * sizeof(double) + 10 * sizeof(float));
   b += static_cast<size_t>(n_rays) * 4 * sizeof(float) * cfg->n_sources;
   // cell-order storage of the particles (on by default): second copies, two order maps, keys, ranks, sources and
