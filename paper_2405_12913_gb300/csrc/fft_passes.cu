@@ -276,14 +276,17 @@ __device__ __forceinline__ void forward_lines(C2 (&v)[32], const Addr& at, const
 }
 
 // Inverse of forward_lines (unnormalised): v[k2] = X[k1 + R1 k2] of pair lane / R1, real and imaginary parts swapped
-// -> v[p R1 + slot<R1>(n2)] = x[lane + 32 n2] of pair p, still swapped.
-template <int R1, class Addr>
-__device__ __forceinline__ void inverse_lines(C2 (&v)[32], const Addr& at, const float2* __restrict__ tw, int lane) {
-  constexpr int P = Cfg<R1>::P;
+// -> v[p R1 + slot<R1>(n2)] = x[lane + 32 n2] of pair p, still swapped.  The first half works in registers only.
+template <int R1>
+__device__ __forceinline__ void inverse_first(C2 (&v)[32], const float2* __restrict__ tw, int lane) {
   dft<32, 0>(v);
   const float2* __restrict__ ti = tw + (R1 == 32 ? 0 : R1 * 32);
 #pragma unroll
   for (int n1 = 1; n1 < 32; ++n1) v[slot<32>(n1)] = twiddled(v[slot<32>(n1)], __ldg(ti + n1 * 32 + lane));
+}
+template <int R1, class Addr>
+__device__ __forceinline__ void inverse_second(C2 (&v)[32], const Addr& at, int lane) {
+  constexpr int P = Cfg<R1>::P;
   const int pb = lane / R1, k1 = lane % R1;
   __syncwarp();
 #pragma unroll
@@ -334,8 +337,9 @@ __global__ void __launch_bounds__(128, 3)
 #pragma unroll 1
   for (int p = 0; p < P; ++p) {
     float* dst = out + (g0 + p) * 4 * static_cast<int64_t>(row_out);
-#pragma unroll 1
-    for (int j = lane; j <= N / 4; j += 32) {
+#pragma unroll(N / 128 < 4 ? N / 128 : 4)
+    for (int t = 0; t < N / 128; ++t) {
+      const int j = lane + 32 * t;
       C2 a[2], b[2];
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
@@ -352,6 +356,11 @@ __global__ void __launch_bounds__(128, 3)
       *reinterpret_cast<float4*>(q + row_out) = make_float4(br0.x, br1.x, bi0.x, bi1.x);
       *reinterpret_cast<float4*>(q + 2 * row_out) = make_float4(ar0.y, ar1.y, ai0.y, ai1.y);
       *reinterpret_cast<float4*>(q + 3 * row_out) = make_float4(br0.y, br1.y, bi0.y, bi1.y);
+    }
+    if (lane < 4) {  // k = n/2 of the four rows
+      const C2 x = lds(at.natural(p, N / 2));
+      const float2 v2 = unpack(lane & 1 ? x.im : x.re);
+      *reinterpret_cast<float4*>(dst + lane * row_out + N) = make_float4(lane & 2 ? v2.y : v2.x, 0.f, 0.f, 0.f);
     }
   }
 }
@@ -412,7 +421,8 @@ __global__ void __launch_bounds__(128, 3)
   C2 v[32];
 #pragma unroll
   for (int k2 = 0; k2 < 32; ++k2) v[k2] = swapped(lds(at.natural(pb, k1 + R1 * k2)));
-  inverse_lines<R1>(v, at, tw, lane);
+  inverse_first<R1>(v, tw, lane);
+  inverse_second<R1>(v, at, lane);
   float* __restrict__ dst = f.out[blockIdx.y] + g0 * 4 * N;
 #pragma unroll
   for (int p = 0; p < P; ++p)
@@ -601,49 +611,63 @@ __global__ void __launch_bounds__(Cfg<R1>::Threads, Cfg<R1>::Blocks)
 }
 
 // ---- x-pass -------------------------------------------------------------------------------------------------
+// Learned factor of |k|, linearly interpolated, 1 beyond the table (without branches).
 __device__ __forceinline__ float learned_factor(const FftSet& s, float kmag) {
   const float t = kmag * s.g_inv_dk;
-  if (t >= static_cast<float>(s.g_nk - 1)) return 1.f;
-  const int i = static_cast<int>(t);
+  const int i = min(static_cast<int>(t), s.g_nk - 2);
   const float w = t - static_cast<float>(i);
-  return __ldg(s.g + i) * (1.f - w) + __ldg(s.g + i + 1) * w;
+  const float g = __ldg(s.g + i) * (1.f - w) + __ldg(s.g + i + 1) * w;
+  return t >= static_cast<float>(s.g_nk - 1) ? 1.f : g;
 }
 
 struct XJobs {
   CUtensorMap in, out[4];
   FftSet set[2];
-  int jobs;
+  int sets;
 };
 
-// One block per (ky, 8 kz) and output: forward along x, Green's function x filter x i [x d_x], inverse along x.
+// One block per (ky, 8 kz) and filter set: forward along x, Green's function x filter x i, then inverse along x of the
+// x component and of V.  Bound by issue and latency (three transforms on one tile's copies: 5000 instructions a warp;
+// 3.15 ms at 1024^3 for 13.1 GB, 0.61 of the copy rate).  Between the two inverses the spectrum waits in registers
+// (kKeep of a lane's 32 pairs) and in a stash beside the tile: with 255 registers a thread and 113 KB, two blocks of four
+// warps per SM.  Other places for it were slower: made again by a second block (three blocks of 168 registers per SM)
+// 3.77 ms, kept in the V spectrum's own lines in L2 3.85 ms.
+constexpr int kKeep = 9;
+template <int R1>
+struct XCfg {
+  static constexpr int Stash = 32 - kKeep;
+  static constexpr int Bytes = Cfg<R1>::TileBytes + Cfg<R1>::W * Stash * 512 + 1024;
+};
+
 template <int R1, bool LEARNED>
-__global__ void __launch_bounds__(Cfg<R1>::Threads, Cfg<R1>::Blocks)
+__global__ void __launch_bounds__(Cfg<R1>::Threads, 8 / Cfg<R1>::W)
     fft_x_kernel(const __grid_constant__ XJobs jobs, const float2* __restrict__ tw, int blocks_kz, float kf, float scale,
                  int* __restrict__ err) {
   using C = Cfg<R1>;
   using T = Tile<R1>;
-  constexpr int N = C::N;
+  constexpr int N = C::N, S = XCfg<R1>::Stash;
   extern __shared__ unsigned char raw[];
   __shared__ uint64_t bar;
   const uint32_t buf = tile_buffer(raw);
-  const unsigned tile = blockIdx.x / static_cast<unsigned>(jobs.jobs);
-  const int job = blockIdx.x - tile * jobs.jobs;
+  const unsigned tile = blockIdx.x / static_cast<unsigned>(jobs.sets);
+  const int set = blockIdx.x - tile * jobs.sets;
   // 16 consecutive tiles share a region: ky mod 16 fastest
   const unsigned region = tile >> 4;
   const int kg = region / blocks_kz, kb = region - kg * blocks_kz, ky = kg * 16 + (tile & 15);
   if (!fetch_tile<R1>(buf, &bar, err, [&](uint32_t d, uint32_t b) { T::load_line(d, &jobs.in, ky, kb, b); })) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const TileAddr at{buf, warp * C::P};
-  C2 v[32];
-#pragma unroll
-  for (int p = 0; p < C::P; ++p)
-#pragma unroll
-    for (int m = 0; m < R1; ++m) v[p * R1 + m] = lds(at(p, lane + 32 * m));
-  forward_lines<R1>(v, at, tw, lane);
+  const uint32_t stash = buf + C::TileBytes + warp * (S * 512) + lane * 16;
+  const int pb = lane / R1, k1 = lane % R1;
+  C2 u[32], keep[kKeep];
   {
-    const FftSet& s = jobs.set[job >> 1];
-    const bool with_dx = (job & 1) == 0;
-    const int pb = lane / R1, k1 = lane % R1;
+    C2 v[32];
+#pragma unroll
+    for (int p = 0; p < C::P; ++p)
+#pragma unroll
+      for (int m = 0; m < R1; ++m) v[p * R1 + m] = lds(at(p, lane + 32 * m));
+    forward_lines<R1>(v, at, tw, lane);
+    const FftSet& s = jobs.set[set];
     const int kz0 = kb * 8 + 2 * (warp * C::P + pb);
     const float kyf = kf * (ky < N / 2 ? ky : ky - N), kza = kf * kz0, kzb = kf * (kz0 + 1);
     const float k2a = kyf * kyf + kza * kza, k2b = kyf * kyf + kzb * kzb;
@@ -651,40 +675,66 @@ __global__ void __launch_bounds__(Cfg<R1>::Threads, Cfg<R1>::Blocks)
     const float ca = wy * __ldg(s.wz + min(kz0, N / 2)), cb = wy * __ldg(s.wz + min(kz0 + 1, N / 2));
     const float* __restrict__ wx = s.wxy + k1;
     const u64 k2ab = pack(k2a, k2b), cab = pack(ca, cb), neg = both(-1.f);
+    auto k_squared = [&](int k2, float kfx) {
+      const int kx = k1 + R1 * k2;
+      const u64 kxf = both(kfx * (k2 < 16 ? kx : kx - N));
+      return fma2(kxf, kxf, k2ab);
+    };
 #pragma unroll
     for (int k2 = 0; k2 < 32; ++k2) {
-      const int kx = k1 + R1 * k2;
-      const int nx = k2 < 16 ? kx : kx - N;
-      const float kxf = kf * nx;
-      const u64 q2 = fma2(both(kxf), both(kxf), k2ab);
-      const float2 q = unpack(q2);
+      const float2 q = unpack(k_squared(k2, kf));
       const float fa = q.x > 0.f ? __fdividef(scale, q.x) : 0.f, fb = __fdividef(scale, q.y);
-      float w = __ldg(wx + R1 * k2);
-      if (with_dx) w *= nx == -(N / 2) ? 0.f : kxf;
-      u64 c = mul2(pack(fa, fb), mul2(both(w), cab));
-      // the learned factor only where its set has one: a uniform branch, in a kernel of its own so that the plain
-      // one stays free of branches
-      if (LEARNED && s.g != nullptr) c = mul2(c, pack(learned_factor(s, sqrtf(q.x)), learned_factor(s, sqrtf(q.y))));
+      const u64 c = mul2(pack(fa, fb), mul2(both(__ldg(wx + R1 * k2)), cab));
       // i c X with the parts swapped for the inverse: (c re, -c im)
-      C2& x = v[slot<32>(k2)];
-      x = {mul2(x.re, c), mul2(x.im, mul2(c, neg))};
+      const C2 x = v[slot<32>(k2)];
+      u[k2] = {mul2(x.re, c), mul2(x.im, mul2(c, neg))};
+    }
+    if (LEARNED && s.g != nullptr) {
+      // |k|^2 again, hidden from the compiler, which else keeps all 64 of them from above
+      float kfl = kf;
+      asm volatile("" : "+f"(kfl));
+#pragma unroll
+      for (int k2 = 0; k2 < 32; ++k2) {
+        const float2 q = unpack(k_squared(k2, kfl));
+        const u64 g = pack(learned_factor(s, sqrtf(q.x)), learned_factor(s, sqrtf(q.y)));
+        u[k2] = {mul2(u[k2].re, g), mul2(u[k2].im, g)};
+      }
     }
   }
-  C2 u[32];
 #pragma unroll
-  for (int k2 = 0; k2 < 32; ++k2) u[k2] = v[slot<32>(k2)];
-  inverse_lines<R1>(u, at, tw, lane);
+  for (int i = 0; i < S; ++i) sts(stash + i * 512, u[i]);
 #pragma unroll
-  for (int p = 0; p < C::P; ++p)
+  for (int i = 0; i < kKeep; ++i) keep[i] = u[S + i];
 #pragma unroll
-    for (int m = 0; m < R1; ++m) sts(at(p, lane + 32 * m), swapped(u[p * R1 + slot<R1>(m)]));
-  fence_async_shared();
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    T::store_line(&jobs.out[job], buf, ky, kb);
-    bulk_commit();
-    bulk_wait_read_all();
+  for (int k2 = 0; k2 < 32; ++k2) {
+    const u64 d = both(derivative(k1 + R1 * k2, N, kf));
+    u[k2] = {mul2(u[k2].re, d), mul2(u[k2].im, d)};
   }
+  inverse_first<R1>(u, tw, lane);
+  inverse_second<R1>(u, at, lane);
+  auto put = [&](int component) {
+#pragma unroll
+    for (int p = 0; p < C::P; ++p)
+#pragma unroll
+      for (int m = 0; m < R1; ++m) sts(at(p, lane + 32 * m), swapped(u[p * R1 + slot<R1>(m)]));
+    fence_async_shared();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      T::store_line(&jobs.out[2 * set + component], buf, ky, kb);
+      bulk_commit();
+    }
+  };
+  put(0);
+#pragma unroll
+  for (int i = 0; i < S; ++i) u[i] = lds(stash + i * 512);
+#pragma unroll
+  for (int i = 0; i < kKeep; ++i) u[S + i] = keep[i];
+  inverse_first<R1>(u, tw, lane);
+  if (threadIdx.x == 0) bulk_wait_read_all();  // the x component has left the tile
+  __syncthreads();
+  inverse_second<R1>(u, at, lane);
+  put(1);
+  if (threadIdx.x == 0) bulk_wait_read_all();
 }
 
 // ---- host ---------------------------------------------------------------------------------------------------
@@ -744,14 +794,14 @@ hrt_status x_pass(const FftPlan& p, double box, double pref, const FftSet& a, co
   const int kb = static_cast<int>(fft_row(C::N) / 8);
   XJobs j{};
   j.in = p.x_in;
-  j.jobs = b ? 4 : 2;
-  for (int i = 0; i < j.jobs; ++i) j.out[i] = p.x_out[i];
+  j.sets = b ? 2 : 1;
+  for (int i = 0; i < 2 * j.sets; ++i) j.out[i] = p.x_out[i];
   j.set[0] = a;
   j.set[1] = b ? *b : a;
   const auto kernel = a.g || (b && b->g) ? fft_x_kernel<R1, true> : fft_x_kernel<R1, false>;
-  HRT_TRY(reserve(kernel, C::TileBytes + 1024));
+  HRT_TRY(reserve(kernel, XCfg<R1>::Bytes));
   const double scale = -pref / (static_cast<double>(C::N) * C::N * C::N);
-  kernel<<<C::N * kb * j.jobs, C::Threads, C::TileBytes + 1024, s>>>(
+  kernel<<<C::N * kb * j.sets, C::Threads, XCfg<R1>::Bytes, s>>>(
       j, p.tw, kb, static_cast<float>(2.0 * M_PI / box), static_cast<float>(scale), p.err);
   HRT_LAUNCHED("fft_x_kernel");
   return HRT_OK;
