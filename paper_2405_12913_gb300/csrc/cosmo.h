@@ -13,16 +13,19 @@ constexpr double kGNewton = 4.30091727e-13;  // (Mpc/h) (100 km/s)^2 / (Msun/h)
 
 struct Cosmo {
   double om;
-  explicit Cosmo(double omega_m) : om(omega_m) {}
+  explicit Cosmo(double omega_m);
   double E(double a) const;
   double chi(double a) const;        // comoving distance of the light front at a
-  double a_of_chi(double chi) const;
+  // inverse of chi; guess (0: none): a scale factor near the answer, such as that of a neighbouring node
+  double a_of_chi(double chi, double guess = 0.0) const;
   double D1(double a) const;         // normalised to 1 at a = 1
   double f(double a) const;          // dln D1 / dln a
   double kick(double a, double b) const;   // int_a^b da / (a E)
   double drift(double a, double b) const;  // int_a^b da / (a^3 E)
  private:
   double growth_integral(double a) const;  // int_0^a da / (a E)^3
+  double panel_;                           // widest quadrature panel in u = sqrt(a)
+  mutable double d1_norm_ = 0.0;           // E(1) times the growth integral at a = 1, once asked for (not thread-safe)
 };
 
 double power_amplitude(double om, double h, double ns, double sigma8);

@@ -561,6 +561,7 @@ static hrt_status plane_table(const hrt_ray_geom& g, double chi_a, double chi_b,
   }
   const int64_t k0 = static_cast<int64_t>(std::ceil((oz + lo) / cell)) - 1;
   const int64_t k1 = static_cast<int64_t>(std::ceil((oz + hi) / cell));
+  double a_near = a_ref;
   for (int64_t kz = k0; kz <= k1; ++kz) {
     const double chi = kz * cell - oz;
     if (!(lo <= chi && chi < hi && chi > 0.0)) continue;
@@ -569,7 +570,8 @@ static hrt_status plane_table(const hrt_ray_geom& g, double chi_a, double chi_b,
     const double r = chi;
     double gw = 1.0;
     if (a_ref > 0.0) {
-      const double a = cosmo.a_of_chi(chi);
+      const double a = cosmo.a_of_chi(chi, a_near);
+      a_near = a;
       gw = cosmo.D1(a) / d1_ref * a_ref / a;
     }
     const double P = r * x2d / cell;
