@@ -776,8 +776,8 @@ hrt_status launch_ray_step_adjoint(const hrt_rays& rays, const float* gx, const 
 // kappa power-spectrum adjoint weights: spec *= W(k) = 2 c lambda_b / count_b for the bin b of the mode
 // (lambda = dL/dP per bin, c = dtheta^4 / Theta^2); modes outside the bins get 0.  The caller then inverts.
 // ---------------------------------------------------------------------------------------------------------
-__global__ void power_adjoint_weight_kernel(float2* __restrict__ spec, int m, double theta_field, int nbins,
-                                            double ln_lmin, double inv_ln_ratio, const double* __restrict__ wbin) {
+__global__ void power_adjoint_weight_kernel(float2* __restrict__ spec, int m, int nbins,
+                                            const __grid_constant__ PowerEdges edges, const double* __restrict__ wbin) {
   const int mzc = m / 2 + 1;
   const int64_t total = static_cast<int64_t>(m) * mzc;
   for (int64_t e = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; e < total;
@@ -785,12 +785,17 @@ __global__ void power_adjoint_weight_kernel(float2* __restrict__ spec, int m, do
     const int ix = static_cast<int>(e / mzc);
     const int iz = static_cast<int>(e - static_cast<int64_t>(ix) * mzc);
     const int nx = ix < m / 2 ? ix : ix - m;
-    const double n2 = static_cast<double>(nx) * nx + static_cast<double>(iz) * iz;
+    const int n2 = nx * nx + iz * iz;
     float w = 0.f;
-    if (n2 > 0.0) {
-      const double ell = 2.0 * M_PI * sqrt(n2) / theta_field;
-      const double t = nbins * (log(ell) - ln_lmin) * inv_ln_ratio + 1e-9;
-      if (t >= 0.0 && t < nbins) w = static_cast<float>(wbin[static_cast<int>(floor(t))]);
+    if (n2 >= edges.first[0] && n2 < edges.first[nbins]) {
+      // the last bin whose first |n|^2 is not above n2
+      int lo = 0, hi = nbins;
+      while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (edges.first[mid] <= n2) lo = mid;
+        else hi = mid;
+      }
+      w = static_cast<float>(wbin[lo]);
     }
     float2 v = spec[e];
     spec[e] = make_float2(w * v.x, w * v.y);
@@ -802,8 +807,8 @@ hrt_status launch_power_adjoint_weight(void* spec, int64_t m, double dtheta, int
   const int64_t total = m * (m / 2 + 1);
   unsigned blocks = blocks_for(total, 256);
   if (blocks > 8 * 152) blocks = 8 * 152;
-  power_adjoint_weight_kernel<<<blocks, 256, 0, s>>>(static_cast<float2*>(spec), static_cast<int>(m), m * dtheta, nbins,
-                                                      std::log(ell_min), 1.0 / std::log(ell_max / ell_min), wbin_dev);
+  power_adjoint_weight_kernel<<<blocks, 256, 0, s>>>(static_cast<float2*>(spec), static_cast<int>(m), nbins,
+                                                      power_edges(m, dtheta, nbins, ell_min, ell_max), wbin_dev);
   HRT_LAUNCHED("power_adjoint_weight_kernel");
   return HRT_OK;
 }

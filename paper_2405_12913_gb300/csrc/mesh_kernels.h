@@ -123,6 +123,12 @@ hrt_status launch_ray_readout(const hrt_rays& rays, float* maps, cudaStream_t s)
 hrt_status launch_rays_init(const hrt_rays& rays, const double* theta0, cudaStream_t s);
 
 // Power-spectrum binning of an m x (m/2+1) half spectrum into sums[3][nbins] (power, ell, count).
+// First |n|^2 of each bin of the power spectrum's rule (hrt_kappa_power), and of the end; m^2 / 2 + 1 if none.
+struct PowerEdges {
+  static constexpr int kMaxBins = 256;
+  int first[kMaxBins + 1];
+};
+PowerEdges power_edges(int64_t m, double dtheta, int nbins, double ell_min, double ell_max);
 hrt_status launch_power_bin(const void* spec, int64_t m, double dtheta, int nbins, double ell_min, double ell_max,
                             double* sums, cudaStream_t s);
 

@@ -372,51 +372,156 @@ hrt_status launch_rays_init(const hrt_rays& rays, const double* theta0, cudaStre
 
 // ---------------------------------------------------------------------------------------------------------
 // Power-spectrum binning of the m x (m/2+1) half spectrum of kappa.  Column kz = 1..m/2-1 stands for two
-// modes (n and -n); kz = 0 and kz = m/2 for one.  The bin of a mode is decided in FP64 exactly as stated in
-// the header.  Per-block shared accumulators, then one FP64 atomic per bin and block into sums[3][nbins].
+// modes (n and -n); kz = 0 and kz = m/2 for one.  The bin rule of the header is increasing in |n|^2, an integer, so the
+// host finds each bin's first |n|^2 with it (FP64) and the kernel compares integers.
+//
+// Bound by latency and the few FP64 lanes of this part: an FP64 logarithm and square root and three FP64 shared-memory
+// atomics per mode, most lanes of a warp on the same bin, took 880 us at m = 2048.  A warp now takes 256 columns of
+// the rows nx and -nx, whose geometry is the same; a lane's modes climb through the bins, so it adds in registers and
+// goes to shared memory when its bin changes (rarely) and, after a sum over the warp, at the end.  |n| is a float
+// square root with its residual (2^-46); the power is summed in FP64.
 // ---------------------------------------------------------------------------------------------------------
-__global__ void power_bin_kernel(const float2* __restrict__ spec, int m, double theta_field, double p_norm,
-                                 int nbins, double ln_lmin, double inv_ln_ratio, double* __restrict__ sums) {
+constexpr int kBinColumns = 256;
+
+__global__ void __launch_bounds__(256) power_bin_kernel(const float2* __restrict__ spec, int m, double ell_scale,
+                                                        double p_norm, int nbins,
+                                                        const __grid_constant__ PowerEdges edges,
+                                                        double* __restrict__ sums) {
   extern __shared__ double sh[];  // [3][nbins]
+  __shared__ int edge[PowerEdges::kMaxBins + 1];
   for (int i = threadIdx.x; i < 3 * nbins; i += blockDim.x) sh[i] = 0.0;
+  for (int i = threadIdx.x; i <= nbins; i += blockDim.x) edge[i] = edges.first[i];
   __syncthreads();
-  const int mzc = m / 2 + 1;
-  const int64_t total = static_cast<int64_t>(m) * mzc;
-  for (int64_t e = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; e < total;
-       e += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    int ix = static_cast<int>(e / mzc);
-    int iz = static_cast<int>(e - static_cast<int64_t>(ix) * mzc);
-    int nx = ix < m / 2 ? ix : ix - m;
-    double n2 = static_cast<double>(nx) * nx + static_cast<double>(iz) * iz;
-    if (n2 <= 0.0) continue;
-    double ell = 2.0 * M_PI * sqrt(n2) / theta_field;
-    double t = nbins * (log(ell) - ln_lmin) * inv_ln_ratio + 1e-9;
-    if (!(t >= 0.0) || t >= nbins) continue;
-    int b = static_cast<int>(floor(t));
-    float2 v = spec[e];
-    double w = (iz == 0 || iz == m / 2) ? 1.0 : 2.0;
-    double pw = (static_cast<double>(v.x) * v.x + static_cast<double>(v.y) * v.y) * p_norm;
-    atomicAdd(sh + b, w * pw);
-    atomicAdd(sh + nbins + b, w * ell);
-    atomicAdd(sh + 2 * nbins + b, w);
+  const int mzc = m / 2 + 1, segments = (mzc + kBinColumns - 1) / kBinColumns, lane = threadIdx.x & 31;
+  const int task = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int nx = task / segments, z0 = (task - nx * segments) * kBinColumns + lane;
+  if (nx <= m / 2) {
+    const bool two = nx > 0 && nx < m / 2;
+    const float2* __restrict__ row = spec + static_cast<int64_t>(nx) * mzc;
+    const float2* __restrict__ mirror = spec + static_cast<int64_t>(m - nx) * mzc;
+    const float2 none = make_float2(0.f, 0.f);
+    float2 u[kBinColumns / 32], v[kBinColumns / 32];
+#pragma unroll
+    for (int i = 0; i < kBinColumns / 32; ++i) {
+      const int iz = z0 + 32 * i;
+      u[i] = iz < mzc ? __ldg(row + iz) : none;
+      v[i] = two && iz < mzc ? __ldg(mirror + iz) : none;
+    }
+    // the bin below the first mode's: the last whose first |n|^2 is not above it, -1 below all
+    int bin = -1;
+    {
+      const int n2 = nx * nx + z0 * z0;
+      for (int lo = 0, hi = nbins; lo <= hi;) {
+        const int mid = (lo + hi) >> 1;
+        if (edge[mid] <= n2) {
+          bin = mid;
+          lo = mid + 1;
+        } else {
+          hi = mid - 1;
+        }
+      }
+    }
+    double power = 0.0;
+    float ell_hi = 0.f, ell_lo = 0.f;
+    int count = 0;
+    auto flush = [&] {
+      if (count > 0 && bin >= 0 && bin < nbins) {
+        atomicAdd(sh + bin, power * p_norm);
+        atomicAdd(sh + nbins + bin, (static_cast<double>(ell_hi) + ell_lo) * ell_scale);
+        atomicAdd(sh + 2 * nbins + bin, static_cast<double>(count));
+      }
+      power = 0.0;
+      ell_hi = ell_lo = 0.f;
+      count = 0;
+    };
+#pragma unroll
+    for (int i = 0; i < kBinColumns / 32; ++i) {
+      const int iz = z0 + 32 * i;
+      const int n2 = nx * nx + iz * iz;
+      if (iz >= mzc || n2 == 0) continue;
+      if (bin < nbins && n2 >= edge[bin + 1]) {
+        flush();
+        do ++bin;
+        while (bin < nbins && n2 >= edge[bin + 1]);
+      }
+      const int each = iz == 0 || iz == m / 2 ? 1 : 2, modes = two ? 2 * each : each;
+      double pw = static_cast<double>(u[i].x) * u[i].x + static_cast<double>(u[i].y) * u[i].y;
+      if (two) pw += static_cast<double>(v[i].x) * v[i].x + static_cast<double>(v[i].y) * v[i].y;
+      power += each == 2 ? 2.0 * pw : pw;
+      count += modes;
+      // modes |n| as hi + lo, added with the rounding error kept (modes is a power of two)
+      const float a = static_cast<float>(n2), rest = static_cast<float>(n2 - static_cast<int>(a));
+      const float s = sqrtf(a), corr = (__fmaf_rn(-s, s, a) + rest) / (2.f * s);
+      const float x = s * modes, sum = ell_hi + x, back = sum - ell_hi;
+      ell_lo += ((ell_hi - (sum - back)) + (x - back)) + corr * modes;
+      ell_hi = sum;
+    }
+    // what is left of each bin, summed over the warp's lanes that hold it
+    unsigned left = __ballot_sync(0xffffffffu, count > 0 && bin >= 0 && bin < nbins);
+    const double ell = (static_cast<double>(ell_hi) + ell_lo) * ell_scale;
+    while (left) {
+      const int leader = __ffs(left) - 1;
+      const int leading = __shfl_sync(0xffffffffu, bin, leader);  // by every lane: not behind a short circuit
+      const bool mine = ((left >> lane) & 1u) && bin == leading;
+      double p = mine ? power * p_norm : 0.0, e = mine ? ell : 0.0;
+      int c = mine ? count : 0;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        p += __shfl_xor_sync(0xffffffffu, p, o);
+        e += __shfl_xor_sync(0xffffffffu, e, o);
+        c += __shfl_xor_sync(0xffffffffu, c, o);
+      }
+      if (lane == leader) {
+        atomicAdd(sh + bin, p);
+        atomicAdd(sh + nbins + bin, e);
+        atomicAdd(sh + 2 * nbins + bin, static_cast<double>(c));
+      }
+      left &= ~__ballot_sync(0xffffffffu, mine);
+    }
   }
   __syncthreads();
   for (int i = threadIdx.x; i < 3 * nbins; i += blockDim.x)
     if (sh[i] != 0.0) atomicAdd(sums + i, sh[i]);
 }
 
+PowerEdges power_edges(int64_t m, double dtheta, int nbins, double ell_min, double ell_max) {
+  const double theta_field = m * dtheta, ln_lmin = std::log(ell_min), inv_ln_ratio = 1.0 / std::log(ell_max / ell_min);
+  const int64_t none = m * m / 2 + 1;  // above every |n|^2
+  auto rule = [&](int64_t n2) {
+    return nbins * (std::log(2.0 * M_PI * std::sqrt(static_cast<double>(n2)) / theta_field) - ln_lmin) * inv_ln_ratio + 1e-9;
+  };
+  PowerEdges e{};
+  for (int b = 0; b <= nbins; ++b) {
+    // next to where the rule's inverse puts it, else (its rounding, or an overflow) by bisection
+    const double ell = std::exp(ln_lmin + (b - 1e-9) / (nbins * inv_ln_ratio)), n = ell * theta_field / (2.0 * M_PI);
+    int64_t lo = 0, hi = none;  // the rule fails at lo and holds at hi, or hi is past the end
+    if (std::isfinite(inv_ln_ratio)) {
+      if (n * n < static_cast<double>(none)) {
+        const int64_t c = static_cast<int64_t>(n * n);
+        if (c > 1 && !(rule(c - 1) >= b)) lo = c - 1;
+        if (c + 2 < none && rule(c + 2) >= b) hi = c + 2;
+      }
+      while (hi - lo > 1) {
+        const int64_t c = lo + (hi - lo) / 2;
+        if (rule(c) >= b) hi = c;
+        else lo = c;
+      }
+    }
+    e.first[b] = static_cast<int>(hi);
+  }
+  return e;
+}
+
 hrt_status launch_power_bin(const void* spec, int64_t m, double dtheta, int nbins, double ell_min, double ell_max,
                             double* sums, cudaStream_t s) {
   HRT_CUDA(cudaMemsetAsync(sums, 0, 3 * nbins * sizeof(double), s));
-  double theta_field = m * dtheta;
+  const double theta_field = m * dtheta;
   // |FFT|^2 dtheta^4 / Theta^2
-  double p_norm = dtheta * dtheta * dtheta * dtheta / (theta_field * theta_field);
-  int64_t total = m * (m / 2 + 1);
-  unsigned blocks = blocks_for(total, 256);
-  if (blocks > 4 * 152) blocks = 4 * 152;
-  power_bin_kernel<<<blocks, 256, 3 * nbins * sizeof(double), s>>>(
-      static_cast<const float2*>(spec), static_cast<int>(m), theta_field, p_norm, nbins, std::log(ell_min),
-      1.0 / std::log(ell_max / ell_min), sums);
+  const double p_norm = dtheta * dtheta * dtheta * dtheta / (theta_field * theta_field);
+  const int64_t warps = (m / 2 + 1) * ((m / 2 + 1 + kBinColumns - 1) / kBinColumns);
+  power_bin_kernel<<<blocks_for(warps, 8), 256, 3 * nbins * sizeof(double), s>>>(
+      static_cast<const float2*>(spec), static_cast<int>(m), 2.0 * M_PI / theta_field, p_norm, nbins,
+      power_edges(m, dtheta, nbins, ell_min, ell_max), sums);
   HRT_LAUNCHED("power_bin_kernel");
   return HRT_OK;
 }
