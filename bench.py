@@ -33,7 +33,7 @@ KERNEL_SOURCES = {
     "ray_step": ["ray_kernels.cu", "mesh_kernels.h"],
     "kick_drift": ["mesh_kernels.cu"],
     "cic_scatter": ["mesh_kernels.cu"],
-    "kspace": ["mesh_kernels.cu", "fft_passes.cu", "tma.h"],
+    "kspace": ["mesh_kernels.cu", "fft_passes.cu", "fft_passes.cuh", "tma.h"],
 }
 
 
@@ -214,7 +214,7 @@ def algorithmic_bytes(W):
 
 def own_fft(W):
     """Whether the library's own FFT passes run the Poisson solve of this mesh (else cuFFT and the k-space kernel)."""
-    return W.n_mesh in (256, 512, 1024)
+    return W.n_mesh in (64, 96, 128, 192, 256, 384, 512, 768, 1024)
 
 
 # ----------------------------------------------------------------------------------------------- GPU arm

@@ -305,13 +305,13 @@ struct hrt_pm {
   hrt::KspaceCallbackInfo* cb_info = nullptr;  // device: [0] particle fields, [1] ray fields
   size_t work_bytes = 0;
   // split path (the default where supported): the library's own FFT passes along z, y and x (fft_passes.h).  Their
-  // spectra lie in rho_hat, grad_hat and split_hat (1, or 3 with ray fields).
-  bool split = false, have_split = false;
+  // spectra lie in rho_hat, grad_hat and split_hat (split_spectra).
+  bool split = false;
   hrt::FftPlan fft;
   float2* twiddles = nullptr;
   void* split_hat = nullptr;
   int* xerr = nullptr;      // device error word of the kernels that wait for TMA copies (FFT passes, tiled deposit)
-  bool last_split = false;  // the last solve took the split path, which leaves no 3D spectrum in rho_hat
+  bool last_split = false;  // the last solve took the split path: rho_hat holds no 3D spectrum
 };
 
 namespace hrt {
@@ -319,9 +319,12 @@ namespace hrt {
 static size_t spectrum_bytes(int64_t n) { return static_cast<size_t>(n) * n * (n / 2 + 1) * sizeof(float2); }
 // Bytes of one spectrum buffer: the half spectrum, or the padded layout of the FFT passes where they exist.
 static size_t spectrum_alloc(int64_t n) { return fft_supported(n) ? fft_spectrum_bytes(n) : spectrum_bytes(n); }
+// Sides whose path the caller chooses (hrt_pm_set_split) and where a split solve leaves no spectrum to copy out.
+static bool split_side(int64_t n) { return n == 256 || n == 512 || n == 1024; }
 // Spectra the FFT passes need beyond the 4 (6 with ray fields) of the 3D path: the transformed density, two spectra
-// per filter set out of the x-pass and all fields but the first between the inverse passes.
-static int split_spectra(int32_t n_ray) { return n_ray > 0 ? 3 : 1; }
+// per filter set out of the x-pass and the fields between the inverse passes, the first of them in place of the
+// density where its spectrum is not asked for later.
+static int split_spectra(int64_t n, int32_t n_ray) { return (n_ray > 0 ? 3 : 1) + (split_side(n) ? 0 : 1); }
 
 static bool fusable(int64_t n) { return n >= 8 && n <= 1024 && (n & (n - 1)) == 0; }
 
@@ -357,7 +360,7 @@ static void pm_set_work(hrt_pm* pm) {
 // Buffers, twiddles and tensor maps of the FFT passes.
 static hrt_status pm_make_split(hrt_pm* pm) {
   const size_t sp = spectrum_alloc(pm->n);
-  HRT_TRY(device_alloc(&pm->split_hat, sp * split_spectra(pm->n_ray), pm->stream, "spectra of the FFT passes"));
+  HRT_TRY(device_alloc(&pm->split_hat, sp * split_spectra(pm->n, pm->n_ray), pm->stream, "spectra of the FFT passes"));
   std::vector<float2> tw;
   fft_twiddles(pm->n, tw);
   HRT_TRY(device_alloc(reinterpret_cast<void**>(&pm->xerr), sizeof(int), pm->stream, "FFT pass error word"));
@@ -367,15 +370,17 @@ static hrt_status pm_make_split(hrt_pm* pm) {
   // the host vector must outlive the copy
   HRT_CUDA(cudaStreamSynchronize(pm->stream));
   const int n_mid = pm->n_ray > 0 ? 4 : 2, fields = 3 + pm->n_ray;
-  void *mid[4], *rest[kFftMaxFields - 1];
+  void *mid[4], *out[kFftMaxFields];
   char* pool[2] = {static_cast<char*>(pm->grad_hat), static_cast<char*>(pm->split_hat)};
-  for (int i = 0; i < n_mid; ++i) mid[i] = pool[0] + i * sp;
-  for (int i = 1; i < fields; ++i) {
-    const int k = n_mid + i - 1;
-    rest[i - 1] = k < fields ? pool[0] + k * sp : pool[1] + (k - fields) * sp;
-  }
-  HRT_TRY(fft_plan(pm->fft, pm->n, fields, pm->rho_hat, mid, rest, pm->twiddles, pm->xerr));
-  pm->have_split = pm->split = true;
+  int used = 0;
+  auto next = [&]() -> void* {
+    const int k = used++;
+    return k < fields ? pool[0] + k * sp : pool[1] + (k - fields) * sp;
+  };
+  for (int i = 0; i < n_mid; ++i) mid[i] = next();
+  for (int i = 0; i < fields; ++i) out[i] = i == 0 && split_side(pm->n) ? pm->rho_hat : next();
+  HRT_TRY(fft_plan(pm->fft, pm->n, fields, pm->rho_hat, mid, out, pm->twiddles, pm->xerr));
+  pm->split = true;
   return HRT_OK;
 }
 
@@ -1068,7 +1073,7 @@ hrt_status hrt_pm_set_fused(hrt_pm* pm, int32_t on) {
 
 hrt_status hrt_pm_set_split(hrt_pm* pm, int32_t on) {
   if (!pm) return fail(HRT_ERR_INVALID_ARG, "pm is NULL");
-  if (on && !pm->have_split) return fail(HRT_ERR_INVALID_ARG, "the split path needs a mesh side of 256, 512 or 1024");
+  if (on && !split_side(pm->n)) return fail(HRT_ERR_INVALID_ARG, "the split path needs a mesh side of 256, 512 or 1024");
   pm->split = on != 0;
   return HRT_OK;
 }
@@ -1649,6 +1654,7 @@ hrt_status hrt_pm_forward_fft(hrt_pm* pm, const float* real, void* out) {
 
 hrt_status hrt_pm_density_spectrum(hrt_pm* pm, void* out) {
   if (!pm || !out) return fail(HRT_ERR_INVALID_ARG, "NULL argument");
+  if (pm->last_split && !split_side(pm->n)) return launch_fft_spectrum(pm->fft, out, pm->stream);
   if (pm->last_split)
     return fail(HRT_ERR_STATE, "the last solve took the split path, which keeps no 3D spectrum (hrt_pm_set_split 0)");
   return cuda_status(cudaMemcpyAsync(out, pm->rho_hat, spectrum_bytes(pm->n), cudaMemcpyDeviceToDevice, pm->stream),
@@ -1677,7 +1683,7 @@ hrt_status hrt_workspace_bytes(const hrt_config* cfg, int64_t n_rays, size_t* by
   const size_t n = cfg->n_mesh, mesh = n * n * n * sizeof(float), np = cfg->n_side * cfg->n_side * cfg->n_side;
   size_t b = 6 * np * sizeof(float) + mesh * (4 + cfg->ray_fields);
   b += spectrum_alloc(cfg->n_mesh) * (1 + 3 + cfg->ray_fields) + 2 * spectrum_bytes(cfg->n_mesh);  // + cuFFT work
-  if (fft_supported(cfg->n_mesh)) b += fft_spectrum_bytes(cfg->n_mesh) * split_spectra(cfg->ray_fields);
+  if (fft_supported(cfg->n_mesh)) b += fft_spectrum_bytes(cfg->n_mesh) * split_spectra(cfg->n_mesh, cfg->ray_fields);
   b += static_cast<size_t>(n_rays) * (2 * sizeof(double) + 10 * sizeof(float));
   b += static_cast<size_t>(n_rays) * 4 * sizeof(float) * cfg->n_sources;
   // cell-order storage of the particles (on by default): second copies, two order maps, keys, ranks, sources and

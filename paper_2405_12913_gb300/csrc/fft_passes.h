@@ -13,7 +13,7 @@
 
 namespace hrt {
 
-// Mesh sides the passes support (n = 32 R1 with R1 in {8, 16, 32}).
+// Mesh sides the passes support: 64, 96, 128, 192, 256, 384, 512, 768, 1024.
 bool fft_supported(int64_t n);
 // kz columns of a row, n/2 + 1 rounded up to the 8 of a tile.
 int64_t fft_row(int64_t n);
@@ -49,8 +49,9 @@ struct FftPlan {
   CUtensorMap y_in, y_out, x_in, x_out[4], iy_in[4], iy_out[kFftMaxFields];
 };
 
-// Fills the plan's maps; half, mid[2 or 4] and out[1 ..] are spectra of fft_spectrum_bytes(n), 128-byte aligned.
-hrt_status fft_plan(FftPlan& p, int64_t n, int fields, void* half, void* const* mid, void* const* out_rest,
+// Fills the plan's maps; half, mid[2 or 4] and out[fields] are spectra of fft_spectrum_bytes(n), 128-byte aligned.  out[0]
+// may be half where its spectrum is not asked for after a solve.
+hrt_status fft_plan(FftPlan& p, int64_t n, int fields, void* half, void* const* mid, void* const* out,
                     const float2* tw, int* err);
 // rho -> (y, z)-transformed density; clear: rho is set to zero once it has been read.
 hrt_status launch_fft_forward(const FftPlan& p, float* rho, bool clear, cudaStream_t s);
@@ -59,5 +60,24 @@ hrt_status launch_fft_x(const FftPlan& p, double box, double pref, const FftSet&
 // grad [3][n^3], and ray [2][n^3] (or nullptr).
 hrt_status launch_fft_inverse_y(const FftPlan& p, double box, bool rays, cudaStream_t s);
 hrt_status launch_fft_inverse_z(const FftPlan& p, float* grad, float* ray, cudaStream_t s);
+// The 3D half spectrum [kx][ky][kz] (complex64) of the density last given to launch_fft_forward; half must still hold it
+// (out[0] is a buffer of its own).
+hrt_status launch_fft_spectrum(const FftPlan& p, void* out, cudaStream_t s);
+
+// The launches for side 32 R1 (fft_passes.cuh).
+template <int R1>
+struct Passes {
+  static hrt_status forward(const FftPlan& p, float* rho, bool clear, cudaStream_t s);
+  static hrt_status x_pass(const FftPlan& p, double box, double pref, const FftSet& a, const FftSet* b, cudaStream_t s);
+  static hrt_status inverse_y(const FftPlan& p, double box, bool rays, cudaStream_t s);
+  static hrt_status inverse_z(const FftPlan& p, float* grad, float* ray, cudaStream_t s);
+  static hrt_status spectrum(const FftPlan& p, void* out, cudaStream_t s);
+};
+extern template struct Passes<2>;
+extern template struct Passes<3>;
+extern template struct Passes<4>;
+extern template struct Passes<6>;
+extern template struct Passes<12>;
+extern template struct Passes<24>;
 
 }  // namespace hrt

@@ -38,7 +38,8 @@ def _solve64(rho, box, pref, deconv, smooth, comps, table=None, k_max=0.0):
     return out
 
 
-@pytest.mark.parametrize("n,rays", [(256, False), (256, True), (512, True), (1024, False)])
+@pytest.mark.parametrize("n,rays", [(64, True), (96, True), (128, False), (192, True), (256, False), (256, True), (384, True),
+                                    (512, True), (768, True), (1024, False)])
 def test_solve_matches_a_64_bit_solve(hrt, n, rays):
     # zero-mean white noise: every mode, the Nyquist planes included, carries the same power.  Rounding of 2 log2(n^3)
     # FP32 butterfly levels plus the multiplier's few factors, each 2^-24 relative to the signal's rms and independent:
@@ -79,3 +80,22 @@ def test_ray_fields_of_a_plan_may_be_left_out(hrt):
         out.append(grad)
         pm.close()
     assert torch.equal(*out)
+
+
+@pytest.mark.parametrize("n", [64, 96, 128, 192, 384, 768])
+def test_density_spectrum_after_a_solve(hrt, n):
+    # sides whose solve always offered the density's 3D spectrum still do, with and without ray fields
+    box = float(n)
+    g = torch.Generator(device="cuda").manual_seed(n)
+    rho = torch.randn(n, n, n, device="cuda", generator=g)
+    want = torch.fft.rfftn(rho.double())
+    f = hrt.make_filter(4.0, 1.0)
+    for rays in (0, 2):
+        pm = hrt.PM(n, box, rays)
+        grad = torch.empty(3, n, n, n, device="cuda")
+        ray = torch.empty(2, n, n, n, device="cuda") if rays else None
+        pm.solve(rho.clone(), 0.45, f, grad, f if rays else None, ray)
+        out = torch.empty(n, n, n // 2 + 1, dtype=torch.complex64, device="cuda")
+        pm.density_spectrum(out)
+        assert (out - want).norm() <= 1e-6 * want.norm()  # log2(n^3) butterfly levels of 2^-24
+        pm.close()
