@@ -12,6 +12,7 @@
 #include "adjoint.h"
 #include "common.h"
 #include "mesh_kernels.h"
+#include "ray_position.cuh"
 
 namespace hrt {
 
@@ -321,14 +322,9 @@ __device__ __forceinline__ NodeField node_field(const float* __restrict__ f, con
   return o;
 }
 
-__device__ __forceinline__ void base_pos(double obs, double r_ref, double theta, double cell, int n, int& i0,
+__device__ __forceinline__ void base_pos(const RayStepParams& p, double obs, double r_ref, double theta, int& i0,
                                          float& f0) {
-  double u = (obs + r_ref * theta) / cell;
-  u -= n * floor(u / n);
-  double fl = floor(u);
-  i0 = static_cast<int>(fl);
-  if (i0 >= n) i0 -= n;
-  f0 = static_cast<float>(u - fl);
+  split_cell(p, line_of_sight_cell(p, obs, r_ref, theta), i0, f0);
 }
 
 // Forward half kick (K, J) at theta, as in the forward kernel.
@@ -339,8 +335,8 @@ __device__ void half_forward(const RayStepParams& p, int j0, int j1, double thx,
   if (j1 <= j0) return;
   int bx, by;
   float fbx, fby;
-  base_pos(p.obs_x, ref_r, thx, p.cell, p.n, bx, fbx);
-  base_pos(p.obs_y, ref_r, thy, p.cell, p.n, by, fby);
+  base_pos(p, p.obs_x, ref_r, thx, bx, fbx);
+  base_pos(p, p.obs_y, ref_r, thy, by, fby);
   const float tx = static_cast<float>(thx), ty = static_cast<float>(thy);
   const float* f[2] = {gx, gy};
   for (int j = j0; j < j1; ++j) {
@@ -366,8 +362,8 @@ __device__ void half_backward(const RayStepParams& p, int j0, int j1, double thx
   int bx = 0, by = 0;
   float fbx = 0.f, fby = 0.f;
   if (active) {
-    base_pos(p.obs_x, ref_r, thx, p.cell, p.n, bx, fbx);
-    base_pos(p.obs_y, ref_r, thy, p.cell, p.n, by, fby);
+    base_pos(p, p.obs_x, ref_r, thx, bx, fbx);
+    base_pos(p, p.obs_y, ref_r, thy, by, fby);
   }
   const float tx = static_cast<float>(thx), ty = static_cast<float>(thy);
   const float inv_cell = static_cast<float>(1.0 / p.cell);
@@ -520,8 +516,8 @@ __device__ void half_forward_tiled(const RayStepParams& p, int j0, int j1, doubl
   if (j1 <= j0) return;
   int bx, by;
   float fbx, fby;
-  base_pos(p.obs_x, ref_r, thx, p.cell, p.n, bx, fbx);
-  base_pos(p.obs_y, ref_r, thy, p.cell, p.n, by, fby);
+  base_pos(p, p.obs_x, ref_r, thx, bx, fbx);
+  base_pos(p, p.obs_y, ref_r, thy, by, fby);
   const float tx = static_cast<float>(thx), ty = static_cast<float>(thy);
   const float* f3[3] = {gx, gy, gz};
   for (int j = j0; j < j1; ++j) {
@@ -550,8 +546,8 @@ __device__ void half_backward_tiled(const RayStepParams& p, int j0, int j1, doub
   int bx = 0, by = 0;
   float fbx = 0.f, fby = 0.f;
   if (active) {
-    base_pos(p.obs_x, ref_r, thx, p.cell, p.n, bx, fbx);
-    base_pos(p.obs_y, ref_r, thy, p.cell, p.n, by, fby);
+    base_pos(p, p.obs_x, ref_r, thx, bx, fbx);
+    base_pos(p, p.obs_y, ref_r, thy, by, fby);
   }
   const float tx = static_cast<float>(thx), ty = static_cast<float>(thy);
   const float inv_cell = static_cast<float>(1.0 / p.cell);

@@ -178,18 +178,24 @@ static hrt_status build_ray_params(const hrt_ray_geom& g, double chi_from, doubl
     }
   }
   p.cell = cell;
+  p.inv_cell = 1.0 / cell;
+  p.inv_n = 1.0 / static_cast<double>(g.n);
   p.box = g.box;
   p.obs_x = g.observer[0];
   p.obs_y = g.observer[1];
+  p.fixed_obs_x = std::ldexp(p.obs_x / cell, 32);
+  p.fixed_obs_y = std::ldexp(p.obs_y / cell, 32);
   p.drift_d = (chi_to - chi_from) / (kCLight * chi_mid * chi_mid);
   p.drift = static_cast<float>(p.drift_d);
   int total = 0;
   double a_near = a_ref;
+  p.r_lo = p.r_hi = chi_mid;
   const double lo[2] = {chi_from, chi_mid}, hi[2] = {chi_mid, chi_to};
   for (int h = 0; h < 2; ++h) {
     int cnt = half_shell_count(lo[h], hi[h], g.samples_per_cell, cell);
     double hh = (hi[h] - lo[h]) / cnt;
     p.ref_r[h] = lo[h] + 0.5 * hh;
+    p.fixed_r[h] = std::ldexp(p.ref_r[h] / cell, 32);
     int kept = 0;
     for (int j = 0; j < cnt; ++j) {
       double chi = lo[h] + (j + 0.5) * hh;
@@ -202,6 +208,8 @@ static hrt_status build_ray_params(const hrt_ray_geom& g, double chi_from, doubl
         gw = cosmo.D1(a) / d1_ref * a_ref / a;
       }
       double r = chi;
+      p.r_lo = std::min(p.r_lo, r);
+      p.r_hi = std::max(p.r_hi, r);
       double c = -(2.0 / kCLight) * hh * r * gw;
       p.dr[total] = static_cast<float>((r - p.ref_r[h]) / cell);
       p.cw[total] = static_cast<float>(c);
@@ -1707,6 +1715,7 @@ hrt_status hrt_destroy(hrt_ctx* ctx) {
   tape_free(ctx);
   int device = 0;
   if (cudaGetDevice(&device) == cudaSuccess) power_plans_release(device, s);
+  ray_planes_release();
   device_free(ctx->disp_alt, s);
   device_free(ctx->mom_alt, s);
   device_free(ctx->order_buf[0], s);

@@ -38,6 +38,7 @@
 
 #include "common.h"
 #include "fft_passes.h"
+#include "packed.cuh"
 #include "tma.h"
 
 namespace hrt {
@@ -45,37 +46,6 @@ namespace hrt {
 namespace {
 
 using namespace tma;
-using u64 = unsigned long long;
-
-// ---- packed pairs -------------------------------------------------------------------------------------------
-__device__ __forceinline__ u64 pack(float a, float b) {
-  u64 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-  return r;
-}
-__device__ __forceinline__ float2 unpack(u64 v) {
-  float2 r;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-  return r;
-}
-__device__ __forceinline__ u64 add2(u64 a, u64 b) {
-  u64 r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ u64 mul2(u64 a, u64 b) {
-  u64 r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ u64 fma2(u64 a, u64 b, u64 c) {
-  u64 r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-__device__ __forceinline__ u64 both(float a) { return pack(a, a); }
-__device__ __forceinline__ u64 sub2(u64 a, u64 b) { return fma2(b, both(-1.f), a); }
-
 // Two complex numbers side by side, 16 bytes in memory: (re, re, im, im).
 struct C2 {
   u64 re, im;

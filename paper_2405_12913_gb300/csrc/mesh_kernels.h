@@ -95,9 +95,12 @@ struct RayStepParams {
   float map_weight;
   float drift;           // (chi_to - chi_from) / (c chi_mid^2), float32 copy for A
   double drift_d;        // the same in FP64 for theta
+  double r_lo, r_hi;     // smallest and largest radius of the kept nodes
   double ref_r[2];       // reference radius of each half shell for the FP64 base position
   double obs_x, obs_y;   // observer transverse position
   double cell, box;
+  double inv_cell, inv_n;  // 1 / cell and 1 / n, rounded
+  double fixed_r[2], fixed_obs_x, fixed_obs_y;  // ref_r / cell, obs / cell in units of 2^-32 cells
   float dr[kMaxRayNodes];   // (r_j - ref_r) / cell
   float cw[kMaxRayNodes];   // c_j
   float cwr[kMaxRayNodes];  // c_j r_j / cell
@@ -118,6 +121,8 @@ struct RayStepParams {
 // gz (the third gradient component) is read only when p.tiled.
 hrt_status launch_ray_step(const hrt_rays& rays, const float* gx, const float* gy, const RayStepParams& p,
                            float* maps, cudaStream_t s, const float* gz = nullptr);
+// Gives back the idle workspace of launch_ray_step on the current device.
+void ray_planes_release();
 hrt_status launch_ray_drift_free(const hrt_rays& rays, double d, cudaStream_t s);
 hrt_status launch_ray_readout(const hrt_rays& rays, float* maps, cudaStream_t s);
 hrt_status launch_rays_init(const hrt_rays& rays, const double* theta0, cudaStream_t s);

@@ -8,10 +8,14 @@
 // interpolation position keeps ~1e-6-cell accuracy at any distance from the observer.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
+#include <mutex>
 
 #include "common.h"
 #include "mesh_kernels.h"
+#include "packed.cuh"
+#include "ray_position.cuh"
 #include "readout.cuh"
 
 namespace hrt {
@@ -21,9 +25,11 @@ struct HalfKick {
   float j00, j01, j10, j11;  // dK/dtheta
 };
 
-__device__ __forceinline__ void base_position(double obs, double r_ref, double theta, double cell, int n,
-                                              int& i0, float& f0, int theta32 = 0) {
-  if (theta32) {
+__device__ __forceinline__ void base_position(const RayStepParams& p, double obs, double r_ref, double theta, int& i0,
+                                              float& f0) {
+  if (p.theta32) {
+    const int n = p.n;
+    const double cell = p.cell;
     // the FP32 ablation: the position and its cell split in single precision
     float uf = (static_cast<float>(obs) + static_cast<float>(r_ref) * static_cast<float>(theta)) / static_cast<float>(cell);
     uf -= static_cast<float>(n) * floorf(uf / static_cast<float>(n));
@@ -34,12 +40,7 @@ __device__ __forceinline__ void base_position(double obs, double r_ref, double t
     f0 = uf - flf;
     return;
   }
-  double u = (obs + r_ref * theta) / cell;
-  u -= n * floor(u / n);
-  double fl = floor(u);
-  i0 = static_cast<int>(fl);
-  if (i0 >= n) i0 -= n;
-  f0 = static_cast<float>(u - fl);
+  split_cell(p, line_of_sight_cell(p, obs, r_ref, theta), i0, f0);
 }
 
 // Wraps k into [0, n): one compare for the usual k within a box of [0, n), the division only beyond.
@@ -72,8 +73,8 @@ __device__ __forceinline__ HalfKick half_kick(const RayStepParams& p, int j0, in
   const int n = p.n;
   int bx, by;
   float fbx, fby;
-  base_position(p.obs_x, ref_r, th_x, p.cell, n, bx, fbx, p.theta32);
-  base_position(p.obs_y, ref_r, th_y, p.cell, n, by, fby, p.theta32);
+  base_position(p, p.obs_x, ref_r, th_x, bx, fbx);
+  base_position(p, p.obs_y, ref_r, th_y, by, fby);
   const float tx = static_cast<float>(th_x), ty = static_cast<float>(th_y);
   const int64_t nn = n;
   for (int j = j0; j < j1; ++j) {
@@ -117,6 +118,191 @@ __device__ __forceinline__ HalfKick half_kick(const RayStepParams& p, int j0, in
     h.j11 += cr * dyy;
   }
   return h;
+}
+
+// ---- node planes --------------------------------------------------------------------------------------------
+// Every ray meets node j at the same z, so the z-interpolation of the two fields at (x, y) is the same for all rays of
+// that cell: 78 of them at 2048^2 rays over 10 degrees and 1024^3 cells.  plane_kernel makes it once per cell of the
+// rays' bounding box into planes [node][y][x] of (d_x phi, d_y phi), 26 MB there, which stay in L2; the ray kernel then
+// gathers four 8-byte corners per node, x fastest as a warp's 16 neighbouring pixels lie, instead of sixteen floats from
+// sixteen columns, with the same arithmetic on the same numbers.  At 2048^2 rays, 60 nodes and 1024^3 cells a step takes
+// 0.60 ms (bounds 21, planes 21, rays 551 us) against 1.57 ms, at 512^2 rays and 256^3 cells 0.12 against 0.31 ms.
+//
+// The box comes from the rays' largest and smallest angles, found on the device in the same step (ray_bounds_kernel).  It
+// is in unwrapped cells and may be wider than the mesh, so that the ray kernel wraps nothing; a ray that leaves it (the
+// angles of the second half shell have moved) reads the fields themselves.
+struct PlaneBox {
+  int x0, y0, rx, ry;  // first cell and extent per axis; rx = 0: no planes in this step
+};
+
+struct RayPlanes {
+  // workspace: ordered keys of max theta_x, max -theta_x, max theta_y, max -theta_y; blocks done; the box
+  unsigned long long* key;
+  unsigned* done;
+  PlaneBox* box;
+  float2* data;
+  int64_t capacity;   // of data, in pairs
+  double r_lo, r_hi;  // smallest and largest node radius
+};
+
+// The bits of a double as an unsigned key of the same order, above 0 for every number; and of its negative.
+__device__ __forceinline__ unsigned long long order_key(unsigned long long b) { return b >> 63 ? ~b : b | (1ull << 63); }
+__device__ __forceinline__ double from_order_key(unsigned long long k) {
+  return __longlong_as_double(static_cast<long long>(k >> 63 ? k ^ (1ull << 63) : ~k));
+}
+
+// Two cells to spare on either side, and the upper corner's.  Extent 0 where that is no sensible number of cells.
+__device__ __forceinline__ void plane_axis(double obs, double t_lo, double t_hi, const RayPlanes& q, double cell, int& first,
+                                           int& extent) {
+  const double a = fmin(q.r_lo * t_lo, q.r_hi * t_lo), b = fmax(q.r_lo * t_hi, q.r_hi * t_hi);
+  const double lo = floor((obs + a) / cell) - 2.0, size = floor((obs + b) / cell) + 4.0 - lo;
+  const bool fine = size >= 1.0 && size <= 65536.0 && fabs(lo) < 1e9;
+  extent = fine ? static_cast<int>(size) : 0;
+  first = fine ? static_cast<int>(lo) : 0;
+}
+
+// Bounds of all angles; the last block to end makes the box of them.  Integer work only per ray: this part has few FP64 lanes.
+__global__ void __launch_bounds__(256) ray_bounds_kernel(const ulonglong2* __restrict__ theta, int64_t nr,
+                                                         const __grid_constant__ RayStepParams p, RayPlanes q) {
+  unsigned long long k[4] = {0, 0, 0, 0};
+  for (int64_t r = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; r < nr;
+       r += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+    const ulonglong2 t = theta[r];
+    k[0] = max(k[0], order_key(t.x));
+    k[1] = max(k[1], order_key(t.x ^ (1ull << 63)));
+    k[2] = max(k[2], order_key(t.y));
+    k[3] = max(k[3], order_key(t.y ^ (1ull << 63)));
+  }
+  __shared__ unsigned long long best[4];
+  if (threadIdx.x < 4) best[threadIdx.x] = 0;
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const unsigned long long other = __shfl_xor_sync(0xffffffffu, k[i], o);
+      k[i] = max(k[i], other);
+    }
+    if ((threadIdx.x & 31) == 0) atomicMax(best + i, k[i]);
+  }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  for (int i = 0; i < 4; ++i) atomicMax(q.key + i, best[i]);
+  __threadfence();
+  if (atomicAdd(q.done, 1u) + 1u != gridDim.x) return;
+  __threadfence();
+  unsigned long long all[4];
+  for (int i = 0; i < 4; ++i) all[i] = atomicMax(q.key + i, 0ull);
+  PlaneBox b;
+  plane_axis(p.obs_x, -from_order_key(all[1]), from_order_key(all[0]), q, p.cell, b.x0, b.rx);
+  plane_axis(p.obs_y, -from_order_key(all[3]), from_order_key(all[2]), q, p.cell, b.y0, b.ry);
+  // fewer rays than cells, or too much to hold: the gather of each ray is the cheaper way
+  const int64_t cells = static_cast<int64_t>(b.rx) * b.ry;
+  if (cells > nr || cells * (p.n1 + p.n2) > q.capacity || b.ry == 0) b.rx = 0;
+  *q.box = b;
+}
+
+// A block makes 32 nodes' planes of 8 x 8 cells: a lane per node, so that a warp reads the columns' z runs as they lie (a
+// thread per cell walking up its column read 32 bytes at a time from rows far apart: 111 us instead of 21 for 60 nodes of 232 x 232
+// cells), eight
+// cells of independent loads per warp, and the planes' rows leave through shared memory.
+constexpr int kPlaneNodes = 32, kPlaneSide = 8;
+
+__global__ void __launch_bounds__(256) plane_kernel(const float* __restrict__ gx, const float* __restrict__ gy,
+                                                    const __grid_constant__ RayStepParams p, RayPlanes q) {
+  __shared__ float2 tile[kPlaneSide * kPlaneSide][kPlaneNodes + 1];
+  const PlaneBox b = *q.box;
+  if (b.rx == 0) return;
+  const int nodes = p.n1 + p.n2, chunks = (nodes + kPlaneNodes - 1) / kPlaneNodes;
+  const int tiles_x = (b.rx + kPlaneSide - 1) / kPlaneSide, tiles_y = (b.ry + kPlaneSide - 1) / kPlaneSide;
+  const int n = p.n, total = tiles_x * tiles_y * chunks, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t plane = static_cast<int64_t>(b.ry) * b.rx;
+  for (int w = blockIdx.x; w < total; w += gridDim.x) {
+    const int t = w / chunks, j0 = (w - t * chunks) * kPlaneNodes, ty = t / tiles_x;
+    const int x0 = (t - ty * tiles_x) * kPlaneSide, y0 = ty * kPlaneSide;
+    const int j = min(j0 + lane, nodes - 1), iz = p.kz[j], jz = iz + 1 == n ? 0 : iz + 1;
+    const float fz = p.fz[j];
+    int cx = (b.x0 + x0 + warp) % n;
+    if (cx < 0) cx += n;
+    float ax[kPlaneSide], ay[kPlaneSide], ux[kPlaneSide], uy[kPlaneSide];
+#pragma unroll
+    for (int y = 0; y < kPlaneSide; ++y) {  // cells past the box: read, not written
+      int cy = (b.y0 + y0 + y) % n;
+      if (cy < 0) cy += n;
+      const int64_t col = (static_cast<int64_t>(cx) * n + cy) * n;
+      ax[y] = __ldg(gx + col + iz);
+      ay[y] = __ldg(gy + col + iz);
+      ux[y] = __ldg(gx + col + jz);
+      uy[y] = __ldg(gy + col + jz);
+    }
+#pragma unroll
+    for (int y = 0; y < kPlaneSide; ++y)
+      tile[y * kPlaneSide + warp][lane] = make_float2(ax[y] + fz * (ux[y] - ax[y]), ay[y] + fz * (uy[y] - ay[y]));
+    __syncthreads();
+    const int xs = min(kPlaneSide, b.rx - x0), ys = min(kPlaneSide, b.ry - y0), count = min(kPlaneNodes, nodes - j0);
+    for (int k = threadIdx.x; k < count * kPlaneSide * kPlaneSide; k += blockDim.x) {
+      const int x = k % kPlaneSide, y = k / kPlaneSide % kPlaneSide, i = k / (kPlaneSide * kPlaneSide);
+      if (x < xs && y < ys)
+        q.data[(j0 + i) * plane + static_cast<int64_t>(y0 + y) * b.rx + x0 + x] = tile[y * kPlaneSide + x][i];
+    }
+    __syncthreads();
+  }
+}
+
+// half_kick on the planes of nodes j0 .. j1; node[j] = (dr, cw, cwr).  The nodes' cells lie between those of the first and
+// the last, so that one look decides for all of them.
+__device__ __forceinline__ HalfKick half_kick_planes(const RayStepParams& p, int j0, int j1, double th_x, double th_y,
+                                                     double ref_r, double fixed_r, const float* __restrict__ gx,
+                                                     const float* __restrict__ gy, const float2* __restrict__ planes,
+                                                     const float4* __restrict__ node, const PlaneBox& b) {
+  if (j1 <= j0) return HalfKick{0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  // cell and fraction from one 32.32 fixed-point number per axis (2^-32 cells; a float's fraction has 2^-24): a single FP64
+  // FMA and a conversion, with the step's constants scaled on the host
+  const long long kx = __double2ll_rd(fma(fixed_r, th_x, p.fixed_obs_x)), ky = __double2ll_rd(fma(fixed_r, th_y, p.fixed_obs_y));
+  const int cx = static_cast<int>(kx >> 32), cy = static_cast<int>(ky >> 32);
+  const float fbx = static_cast<float>(static_cast<unsigned>(kx)) * 0x1p-32f, fby = static_cast<float>(static_cast<unsigned>(ky)) * 0x1p-32f;
+  const int bx = cx - b.x0, by = cy - b.y0;
+  const float tx = static_cast<float>(th_x), ty = static_cast<float>(th_y);
+  auto inside = [&](float dr) {
+    const float px = fbx + dr * tx, py = fby + dr * ty;
+    if (!(fabsf(px) < 65536.f && fabsf(py) < 65536.f)) return false;
+    const int x = bx + static_cast<int>(floorf(px)), y = by + static_cast<int>(floorf(py));
+    return x >= 0 && x + 1 < b.rx && y >= 0 && y + 1 < b.ry;
+  };
+  // (angles that are not finite, or out of the conversion's range, end outside)
+  if (abs(cx + 1) > (1 << 30) || abs(cy + 1) > (1 << 30) || !inside(node[j0].x) || !inside(node[j1 - 1].x))
+    return half_kick(p, j0, j1, th_x, th_y, ref_r, gx, gy);
+  // floor as an integer from the bits of floor + 1.5 2^23 (the conversion unit is slow); the offset of those bits is taken
+  // off here once
+  constexpr float kMagic = 12582912.f;
+  constexpr unsigned kMagicBits = 0x4b400000u;
+  const int plane = b.rx * b.ry;
+  const unsigned offset = static_cast<unsigned>(by * b.rx + bx) - kMagicBits * static_cast<unsigned>(b.rx + 1);
+  const float2* __restrict__ at = planes + static_cast<int64_t>(j0) * plane;
+  // both components of a corner, (d_x phi, d_y phi), side by side
+  u64 k = 0, jx = 0, jy = 0;
+  auto corner = [](const float2* c) { return static_cast<u64>(__ldg(reinterpret_cast<const unsigned long long*>(c))); };
+#pragma unroll 4
+  for (int j = j0; j < j1; ++j, at += plane) {
+    const float4 nd = node[j];
+    const float px = fbx + nd.x * tx, py = fby + nd.x * ty;
+    const float lx = floorf(px), ly = floorf(py);
+    const u64 fx = both(px - lx), fy = both(py - ly);
+    const unsigned e = offset + static_cast<unsigned>(__float_as_int(ly + kMagic)) * static_cast<unsigned>(b.rx) +
+                       static_cast<unsigned>(__float_as_int(lx + kMagic));
+    const float2* __restrict__ q = at + static_cast<int>(e);
+    const u64 c0 = corner(q), c2 = corner(q + 1), c1 = corner(q + b.rx), c3 = corner(q + b.rx + 1);
+    // bilinear value and transverse derivatives (per cell; 1/cell is folded into cwr)
+    const u64 e0 = sub2(c1, c0), e1 = sub2(c3, c2);
+    const u64 v0 = fma2(fy, e0, c0), v1 = fma2(fy, e1, c2), dx = sub2(v1, v0);
+    const u64 v = fma2(fx, dx, v0), dy = fma2(fx, sub2(e1, e0), e0);
+    const u64 cw = both(nd.y), cr = both(nd.z);
+    k = fma2(cw, v, k);
+    jx = fma2(cr, dx, jx);
+    jy = fma2(cr, dy, jy);
+  }
+  const float2 kk = unpack(k), jxx = unpack(jx), jyy = unpack(jy);
+  return {kk.x, kk.y, jxx.x, jyy.x, jxx.y, jyy.y};
 }
 
 // Cell and fraction on a box axis of a sky coordinate (cell i_s, fraction f_s) under sign sgn and a translation
@@ -167,8 +353,8 @@ __device__ __forceinline__ HalfKick half_kick_tiled(const RayStepParams& p, int 
   const int n = p.n;
   int bx, by;
   float fbx, fby;
-  base_position(p.obs_x, ref_r, th_x, p.cell, n, bx, fbx, p.theta32);
-  base_position(p.obs_y, ref_r, th_y, p.cell, n, by, fby, p.theta32);
+  base_position(p, p.obs_x, ref_r, th_x, bx, fbx);
+  base_position(p, p.obs_y, ref_r, th_y, by, fby);
   const float tx = static_cast<float>(th_x), ty = static_cast<float>(th_y);
   const int64_t nn = n;
   for (int j = j0; j < j1; ++j) {
@@ -211,15 +397,33 @@ __device__ __forceinline__ HalfKick half_kick_tiled(const RayStepParams& p, int 
   return h;
 }
 
-// One thread per ray.  __launch_bounds__(128, 1) leaves the register count to the compiler (72 for the direct
-// gather): measured at 2048^2 rays over a 1024^3 mesh, 1.05 ms per step against 1.29 ms with 56 registers, and
-// unrolling the node loop (1.13-1.49 ms) does not help; the loop waits on the latency of its gathers.
-template <bool TILED>
-__global__ void __launch_bounds__(128, 1) ray_step_kernel(double2* __restrict__ theta, float2* __restrict__ eta,
+// One thread per ray.  On the planes the loop is bound by the latency and the issue of its gathers, four 8-byte loads a
+// node: four blocks of 128 per SM (128 registers) and four nodes in flight measured 551 us at 2048^2 rays and 60 nodes,
+// against 643 us with five blocks, 601 us with two nodes in flight, 684 us with eight.  From the fields
+// __launch_bounds__(128, 1) leaves the register count to the compiler (72): 1.05 ms per step against 1.29 ms with 56.
+enum class Gather { kFields, kTiled, kPlanes };
+
+template <Gather G>
+__global__ void __launch_bounds__(128, G == Gather::kPlanes ? 4 : 1) ray_step_kernel(double2* __restrict__ theta, float2* __restrict__ eta,
                                                        float4* __restrict__ Amat, float4* __restrict__ Bmat,
                                                        int64_t nr, const float* __restrict__ gx,
                                                        const float* __restrict__ gy, const __grid_constant__ RayStepParams p,
-                                                       float* __restrict__ maps, const float* __restrict__ gz) {
+                                                       float* __restrict__ maps, const float* __restrict__ gz,
+                                                       RayPlanes planes) {
+  constexpr bool TILED = G == Gather::kTiled;
+  extern __shared__ float4 node[];  // planes: (dr, cw, cwr) of the nodes
+  PlaneBox box{0, 0, 0, 0};
+  if constexpr (G == Gather::kPlanes) {
+    box = *planes.box;
+    for (int j = threadIdx.x; j < p.n1 + p.n2; j += blockDim.x) node[j] = make_float4(p.dr[j], p.cw[j], p.cwr[j], 0.f);
+    __syncthreads();
+  }
+  auto half = [&](int j0, int j1, const double2& t, double ref_r) {
+    if constexpr (TILED) return half_kick_tiled(p, j0, j1, t.x, t.y, ref_r, gx, gy, gz);
+    if constexpr (G == Gather::kPlanes)
+      if (box.rx > 0) return half_kick_planes(p, j0, j1, t.x, t.y, ref_r, p.fixed_r[j0 > 0], gx, gy, planes.data, node, box);
+    return half_kick(p, j0, j1, t.x, t.y, ref_r, gx, gy);
+  };
   int64_t r;
   if (p.tile_w > 0) {
     // 16 x 8 pixel tiles in row-major tile order; a warp covers 16 x 2 neighbouring pixels
@@ -235,8 +439,7 @@ __global__ void __launch_bounds__(128, 1) ray_step_kernel(double2* __restrict__ 
   float2 et = eta[r];
   float4 A = Amat[r], B = Bmat[r];
 
-  HalfKick h = TILED ? half_kick_tiled(p, 0, p.n1, th.x, th.y, p.ref_r[0], gx, gy, gz)
-                     : half_kick(p, 0, p.n1, th.x, th.y, p.ref_r[0], gx, gy);
+  HalfKick h = half(0, p.n1, th, p.ref_r[0]);
   et.x += h.kx;
   et.y += h.ky;
   // B += J A (row-major 2x2: x = 11, y = 12, z = 21, w = 22)
@@ -258,8 +461,7 @@ __global__ void __launch_bounds__(128, 1) ray_step_kernel(double2* __restrict__ 
   A.y += p.drift * B.y;
   A.z += p.drift * B.z;
   A.w += p.drift * B.w;
-  h = TILED ? half_kick_tiled(p, p.n1, p.n1 + p.n2, th.x, th.y, p.ref_r[1], gx, gy, gz)
-            : half_kick(p, p.n1, p.n1 + p.n2, th.x, th.y, p.ref_r[1], gx, gy);
+  h = half(p.n1, p.n1 + p.n2, th, p.ref_r[1]);
   et.x += h.kx;
   et.y += h.ky;
   B.x += h.j00 * A.x + h.j01 * A.z;
@@ -290,16 +492,85 @@ __global__ void __launch_bounds__(128, 1) ray_step_kernel(double2* __restrict__ 
   }
 }
 
+// Workspace of the node planes: stream-ordered from a pool of the library's own, which keeps at most kPlanePoolBytes per
+// device between calls (given back by ray_planes_release).
+constexpr size_t kPlaneBytes = size_t{96} << 20, kPlanePoolBytes = size_t{128} << 20;
+constexpr int kPoolDevices = 16;
+static std::mutex g_plane_mutex;
+static cudaMemPool_t g_plane_pool[kPoolDevices] = {};
+
+static cudaMemPool_t plane_pool() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev >= kPoolDevices) return nullptr;
+  std::lock_guard<std::mutex> lock(g_plane_mutex);
+  if (!g_plane_pool[dev]) {
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t pool = nullptr;
+    if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
+    uint64_t keep = kPlanePoolBytes;
+    cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    g_plane_pool[dev] = pool;
+  }
+  return g_plane_pool[dev];
+}
+
+void ray_planes_release() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev >= kPoolDevices) return;
+  std::lock_guard<std::mutex> lock(g_plane_mutex);
+  if (g_plane_pool[dev]) cudaMemPoolTrimTo(g_plane_pool[dev], 0);
+}
+
+// Rays times nodes from which the three small launches before the step's pay (the gather does about 150 per ns).
+constexpr int64_t kPlaneRays = 1 << 14, kPlaneWork = 1 << 22;
+
 hrt_status launch_ray_step(const hrt_rays& rays, const float* gx, const float* gy, const RayStepParams& p,
                            float* maps, cudaStream_t s, const float* gz) {
   if (rays.n_rays == 0) return HRT_OK;
   if (p.tiled && !gz) return fail(HRT_ERR_INVALID_ARG, "light-cone tiling needs the third gradient component");
-  auto* kernel = p.tiled ? ray_step_kernel<true> : ray_step_kernel<false>;
-  kernel<<<blocks_for(rays.n_rays, 128), 128, 0, s>>>(
+  auto* kernel = p.tiled ? ray_step_kernel<Gather::kTiled> : ray_step_kernel<Gather::kFields>;
+  RayPlanes q{};
+  const int nodes = p.n1 + p.n2;
+  char* work = nullptr;
+  cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+  if (!p.tiled && !p.theta32 && rays.n_rays >= kPlaneRays && rays.n_rays * nodes >= kPlaneWork &&
+      cudaStreamIsCapturing(s, &capturing) == cudaSuccess && capturing == cudaStreamCaptureStatusNone) {
+    // a step without the workspace (or being captured) gathers from the fields
+    const size_t most = static_cast<size_t>(nodes) * rays.n_rays * sizeof(float2);  // no more cells than rays
+    const size_t bytes = most < kPlaneBytes ? most : kPlaneBytes;
+    cudaMemPool_t pool = plane_pool();
+    if (pool && cudaMallocFromPoolAsync(reinterpret_cast<void**>(&work), 256 + bytes, pool, s) == cudaSuccess) {
+      q.key = reinterpret_cast<unsigned long long*>(work);
+      q.done = reinterpret_cast<unsigned*>(work + 32);
+      q.box = reinterpret_cast<PlaneBox*>(work + 48);
+      q.data = reinterpret_cast<float2*>(work + 256);
+      q.capacity = static_cast<int64_t>(bytes / sizeof(float2));
+      q.r_lo = p.r_lo;
+      q.r_hi = p.r_hi;
+      kernel = ray_step_kernel<Gather::kPlanes>;
+    } else {
+      cudaGetLastError();
+      work = nullptr;
+    }
+  }
+  if (work) {
+    HRT_CUDA(cudaMemsetAsync(work, 0, 256, s));
+    ray_bounds_kernel<<<std::min(blocks_for(rays.n_rays, 256), 152u * 8u), 256, 0, s>>>(
+        reinterpret_cast<const ulonglong2*>(rays.theta), rays.n_rays, p, q);
+    plane_kernel<<<152 * 8, 256, 0, s>>>(gx, gy, p, q);
+  }
+  kernel<<<blocks_for(rays.n_rays, 128), 128, work ? nodes * sizeof(float4) : 0, s>>>(
       reinterpret_cast<double2*>(rays.theta), reinterpret_cast<float2*>(rays.eta),
-      reinterpret_cast<float4*>(rays.A), reinterpret_cast<float4*>(rays.B), rays.n_rays, gx, gy, p, maps, gz);
-  HRT_LAUNCHED("ray_step_kernel");
-  return HRT_OK;
+      reinterpret_cast<float4*>(rays.A), reinterpret_cast<float4*>(rays.B), rays.n_rays, gx, gy, p, maps, gz, q);
+  const cudaError_t launched = cudaGetLastError();
+  if (work) cudaFreeAsync(work, s);
+  return cuda_status(launched, "ray_step_kernel");
 }
 
 __global__ void ray_drift_kernel(double2* __restrict__ theta, const float2* __restrict__ eta,
