@@ -502,6 +502,10 @@ static KspaceCallbackInfo callback_info(const hrt_pm* pm, const float* tab, cons
   return ci;
 }
 
+static FftSet fft_set(const hrt_pm* pm, const float* tab, const hrt_filter& f) {
+  return FftSet{tab, tab + pm->n, f.g_table, f.g_nk, f.g_table ? static_cast<float>((f.g_nk - 1) / f.g_kmax) : 0.f};
+}
+
 // before_fields (optional): an event the stream waits for before the C2Rs overwrite grad / ray_grad (work on
 // another stream that still reads the previous fields).  cleared: on the split path the forward z-pass sets rho to
 // zero once it has read it (*cleared tells whether it did), which spares the next deposit its memset.
@@ -523,13 +527,9 @@ static hrt_status pm_solve(hrt_pm* pm, float* rho, double pref, const hrt_filter
       HRT_TRY(launch_fft_forward(pm->fft, rho, cleared != nullptr, pm->stream));
       if (cleared) *cleared = true;
     }
-    auto set = [&](const float* tab, const hrt_filter& flt) {
-      return FftSet{tab, tab + pm->n, flt.g_table, flt.g_nk,
-                    flt.g_table ? static_cast<float>((flt.g_nk - 1) / flt.g_kmax) : 0.f};
-    };
     {
       PhaseScope ps(pc, 4);
-      const FftSet a = set(pm->tab_a, *f), b = rays ? set(pm->tab_b, *fr) : FftSet{};
+      const FftSet a = fft_set(pm, pm->tab_a, *f), b = rays ? fft_set(pm, pm->tab_b, *fr) : FftSet{};
       HRT_TRY(launch_fft_x(pm->fft, pm->box, pref, a, rays ? &b : nullptr, pm->stream));
     }
     PhaseScope ps(pc, 5);
@@ -1302,6 +1302,9 @@ hrt_status hrt_pm_solve_adjoint(hrt_pm* pm, float* grad_bar, double pref, const 
   if (ray_grad_bar) HRT_TRY(check_filter(f_ray));
   HRT_TRY(pm_tables(pm, *f, &pm->tab_a, &pm->key_a));
   if (ray_grad_bar) HRT_TRY(pm_tables(pm, *f_ray, &pm->tab_b, &pm->key_b));
+  // fields of one filter set where the FFT passes run; with ray fields the 3D plans
+  if (pm->split && !ray_grad_bar)
+    return launch_fft_adjoint(pm->fft, pm->box, pref, fft_set(pm, pm->tab_a, *f), grad_bar, rho_bar, pm->stream);
   const size_t sb = spectrum_bytes(pm->n), mb = static_cast<size_t>(pm->n) * pm->n * pm->n;
   char* gh = static_cast<char*>(pm->grad_hat);
   for (int j = 0; j < 3; ++j)

@@ -112,7 +112,20 @@ hrt_status fft_plan(FftPlan& p, int64_t n, int fields, void* half, void* const* 
     HRT_TRY(tile_map(&p.iy_in[i], mid[i], n, true));
   }
   for (int i = 0; i < fields; ++i) HRT_TRY(plane_map(&p.iy_out[i], p.out[i], n));
-  return HRT_OK;
+  // the transposed solve: rows in mid[0] and mid[1]; tiles of the cotangents in the density's place and two fields'
+  void* tiles[3] = {half, out[1], out[2]};
+  FftAdjointPlan& a = p.adjoint;
+  for (int i = 0; i < 2; ++i) {
+    a.rows[i] = static_cast<float*>(mid[i]);
+    HRT_TRY(plane_map(&a.y_in[i], mid[i], n));
+  }
+  for (int i = 0; i < 3; ++i) {
+    HRT_TRY(tile_map(&a.y_out[i], tiles[i], n, true));
+    HRT_TRY(tile_map(&a.x_in[i], tiles[i], n, false));
+  }
+  HRT_TRY(tile_map(&a.x_out, mid[1], n, false));
+  HRT_TRY(tile_map(&a.iy_in, mid[1], n, true));
+  return plane_map(&a.iy_out, mid[0], n);
 }
 
 #define HRT_FFT_SIDE(call)                                                           \
@@ -143,6 +156,11 @@ hrt_status launch_fft_inverse_y(const FftPlan& p, double box, bool rays, cudaStr
 
 hrt_status launch_fft_inverse_z(const FftPlan& p, float* grad, float* ray, cudaStream_t s) {
   HRT_FFT_SIDE(inverse_z(p, grad, ray, s))
+}
+
+hrt_status launch_fft_adjoint(const FftPlan& p, double box, double pref, const FftSet& a, const float* grad_bar, float* rho_bar,
+                              cudaStream_t s) {
+  HRT_FFT_SIDE(adjoint(p, box, pref, a, grad_bar, rho_bar, s))
 }
 
 hrt_status launch_fft_spectrum(const FftPlan& p, void* out, cudaStream_t s) { HRT_FFT_SIDE(spectrum(p, out, s)) }

@@ -299,19 +299,29 @@ __device__ __forceinline__ void inverse_second(C2 (&v)[32], const Addr& at, int 
 }
 
 // ---- z-passes -----------------------------------------------------------------------------------------------
+struct ZFields {
+  const float* in[kFftMaxFields];
+  float* out[kFftMaxFields];
+};
+
+struct ZForward {
+  float* in[2];  // zeroed once read, on request
+  float* out[2];
+};
+
 // A warp takes P groups of four consecutive rows; a group's lines are row 0 + i row 1 and row 2 + i row 3.
 // Forward: bound by memory (8.7 GB, with the zeroing 13 GB at 1024^3).
 template <int R1>
 __global__ void __launch_bounds__(128, 3)
-    fft_z_kernel(float* __restrict__ rho, float* __restrict__ out, const float2* __restrict__ tw, int groups, int row_out,
-                 bool clear) {
+    fft_z_kernel(const __grid_constant__ ZForward f, const float2* __restrict__ tw, int groups, int row_out, bool clear) {
   constexpr int N = 32 * R1, P = Cfg<R1>::P;
   extern __shared__ __align__(16) unsigned char smem[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t g0 = (static_cast<int64_t>(blockIdx.x) * 4 + warp) * P;
   if (g0 >= groups) return;
   const RowAddr<N> at{smem_u32(smem) + warp * (P * N * 16)};
-  float* __restrict__ src = rho + g0 * 4 * N;
+  float* __restrict__ src = f.in[blockIdx.y] + g0 * 4 * N;
+  float* __restrict__ out = f.out[blockIdx.y];
   C2 v[32];
 #pragma unroll
   for (int p = 0; p < P; ++p)
@@ -364,11 +374,6 @@ __global__ void __launch_bounds__(128, 3)
     }
   }
 }
-
-struct ZFields {
-  const float* in[kFftMaxFields];
-  float* out[kFftMaxFields];
-};
 
 // Inverse: the imaginary parts of k = 0 and n/2 do not count, as in any complex-to-real transform.
 template <int R1>
@@ -514,6 +519,25 @@ __device__ __forceinline__ bool fetch_tile(uint32_t buf, uint64_t* bar, int* __r
   return false;
 }
 
+// The next tile into the block's buffer once every warp is done with the last one; phase: its number, from 1.
+template <int R1, class Load>
+__device__ __forceinline__ bool fetch_next(uint32_t buf, uint64_t* bar, uint32_t phase, int* __restrict__ err, Load load) {
+  const uint32_t b = smem_u32(bar);
+  fence_async_shared();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    mbar_expect_tx(b, Cfg<R1>::TileBytes);
+    load(buf, b);
+  }
+  const bool got = mbar_wait(b, phase & 1u);
+  if (__syncthreads_and(got)) return true;
+  if (threadIdx.x == 0) {
+    atomicOr(err, kFftTimeout);
+    mbar_wait(b, phase & 1u);
+  }
+  return false;
+}
+
 __device__ __forceinline__ uint32_t tile_buffer(const unsigned char* raw) {
   const uint32_t a = smem_u32(raw);
   return (a + 1023u) & ~1023u;
@@ -526,18 +550,21 @@ __device__ __forceinline__ float derivative(int k, int n, float kf) {
 }
 
 // ---- y-passes -----------------------------------------------------------------------------------------------
+struct YForward {
+  CUtensorMap in[2], out[2];
+};
+
 // Forward: rows of plane x -> column tile.  One block per (x, 8 kz).
 template <int R1>
 __global__ void __launch_bounds__(Cfg<R1>::Threads, Cfg<R1>::Blocks)
-    fft_y_kernel(const __grid_constant__ CUtensorMap in, const __grid_constant__ CUtensorMap out,
-                 const float2* __restrict__ tw, int blocks_kz, int* __restrict__ err) {
+    fft_y_kernel(const __grid_constant__ YForward f, const float2* __restrict__ tw, int blocks_kz, int* __restrict__ err) {
   using C = Cfg<R1>;
   using T = Tile<R1>;
   extern __shared__ unsigned char raw[];
   __shared__ uint64_t bar;
   const uint32_t buf = tile_buffer(raw);
   const int x = blockIdx.x / blocks_kz, kb = blockIdx.x - x * blocks_kz;
-  if (!fetch_tile<R1>(buf, &bar, err, [&](uint32_t d, uint32_t b) { T::load_plane(d, &in, x, kb, b); })) return;
+  if (!fetch_tile<R1>(buf, &bar, err, [&](uint32_t d, uint32_t b) { T::load_plane(d, &f.in[blockIdx.y], x, kb, b); })) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const TileAddr at{buf, warp * C::P};
   C2 v[32];
@@ -552,7 +579,7 @@ __global__ void __launch_bounds__(Cfg<R1>::Threads, Cfg<R1>::Blocks)
   fence_async_shared();
   __syncthreads();
   if (threadIdx.x == 0) {
-    T::store_column(&out, buf, x, kb);
+    T::store_column(&f.out[blockIdx.y], buf, x, kb);
     bulk_commit();
     bulk_wait_read_all();
   }
@@ -770,6 +797,103 @@ __global__ void __launch_bounds__(Cfg<R1>::Threads, 8 / Cfg<R1>::W)
   if (threadIdx.x == 0) bulk_wait_read_all();
 }
 
+// Transpose of the x-pass for one filter set: out = IFFT_x(-i c (d_x FFT_x(in[0]) + FFT_x(d_y in[1] + d_z in[2]))), the
+// sum of the three cotangents' parts under the conjugate factors.  The first sum waits beside the tile, as in
+// fft_x_kernel, while the x component comes into its place.
+struct XAdjoint {
+  CUtensorMap in[3], out;
+  FftSet set;
+};
+
+template <int R1, bool LEARNED>
+__global__ void __launch_bounds__(Cfg<R1>::Threads, 8 / Cfg<R1>::W)
+    fft_x_adjoint_kernel(const __grid_constant__ XAdjoint f, const float2* __restrict__ tw, int blocks_kz, float kf, float scale,
+                         int* __restrict__ err) {
+  using C = Cfg<R1>;
+  using T = Tile<R1>;
+  constexpr int N = C::N, S = XCfg<R1>::Stash;
+  extern __shared__ unsigned char raw[];
+  __shared__ uint64_t bar;
+  const uint32_t buf = tile_buffer(raw);
+  const unsigned region = blockIdx.x >> 4;
+  const int kg = region / blocks_kz, kb = region - kg * blocks_kz, ky = kg * 16 + (blockIdx.x & 15);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const TileAddr at{buf, warp * C::P};
+  const uint32_t stash = buf + C::TileBytes + warp * (S * 512) + lane * 16;
+  const int lb = C::second(lane), pb = lb / R1, k1 = lb % R1;
+  auto load = [&](const CUtensorMap* m) {
+    return [=](uint32_t d, uint32_t b) { T::load_line(d, m, ky, kb, b); };
+  };
+  C2 v[32], keep[kKeep];
+  if (!fetch_tile<R1>(buf, &bar, err, load(&f.in[1]))) return;
+  const u64 dy = both(derivative(ky, N, kf));
+#pragma unroll
+  for (int p = 0; p < C::P; ++p)
+#pragma unroll
+    for (int m = 0; m < R1; ++m) {
+      const C2 x = lds(at(p, lane + 32 * m));
+      v[p * R1 + m] = {mul2(x.re, dy), mul2(x.im, dy)};
+    }
+  if (!fetch_next<R1>(buf, &bar, 1, err, load(&f.in[2]))) return;
+#pragma unroll
+  for (int p = 0; p < C::P; ++p) {
+    const int kz = kb * 8 + 2 * (warp * C::P + p);
+    const u64 dz = pack(kz == N / 2 ? 0.f : kf * kz, kf * (kz + 1));
+#pragma unroll
+    for (int m = 0; m < R1; ++m) {
+      const C2 x = lds(at(p, lane + 32 * m));
+      C2& y = v[p * R1 + m];
+      y = {fma2(x.re, dz, y.re), fma2(x.im, dz, y.im)};
+    }
+  }
+  forward_lines<R1>(v, at, tw, lane);
+#pragma unroll
+  for (int i = 0; i < S; ++i) sts(stash + i * 512, v[slot<32>(i)]);
+#pragma unroll
+  for (int i = 0; i < kKeep; ++i) keep[i] = v[slot<32>(S + i)];
+  if (!fetch_next<R1>(buf, &bar, 2, err, load(&f.in[0]))) return;
+#pragma unroll
+  for (int p = 0; p < C::P; ++p)
+#pragma unroll
+    for (int m = 0; m < R1; ++m) v[p * R1 + m] = lds(at(p, lane + 32 * m));
+  forward_lines<R1>(v, at, tw, lane);
+  C2 u[32];
+  {
+    const FftSet& s = f.set;
+    const int kz0 = kb * 8 + 2 * (warp * C::P + pb);
+    const float kyf = kf * (ky < N / 2 ? ky : ky - N), kza = kf * kz0, kzb = kf * (kz0 + 1);
+    const float wy = __ldg(s.wxy + ky);
+    const float ca = wy * __ldg(s.wz + min(kz0, N / 2)), cb = wy * __ldg(s.wz + min(kz0 + 1, N / 2));
+    const float* __restrict__ wx = s.wxy + k1;
+    const u64 k2ab = pack(kyf * kyf + kza * kza, kyf * kyf + kzb * kzb), cab = pack(ca, cb), neg = both(-1.f);
+#pragma unroll
+    for (int k2 = 0; k2 < 32; ++k2) {
+      const int kx = k1 + R1 * k2;
+      const u64 kxf = both(kf * (k2 < 16 ? kx : kx - N)), dx = both(derivative(kx, N, kf));
+      const float2 q = unpack(fma2(kxf, kxf, k2ab));
+      const float fa = q.x > 0.f ? __fdividef(scale, q.x) : 0.f, fb = __fdividef(scale, q.y);
+      u64 c = mul2(pack(fa, fb), mul2(both(__ldg(wx + R1 * k2)), cab));
+      if (LEARNED) c = mul2(c, pack(learned_factor(s, sqrtf(q.x)), learned_factor(s, sqrtf(q.y))));
+      const C2 rest = k2 < S ? lds(stash + k2 * 512) : keep[k2 < S ? 0 : k2 - S], x = v[slot<32>(k2)];
+      // -i c X with the parts swapped for the inverse: (-c re, c im)
+      u[k2] = {mul2(fma2(x.re, dx, rest.re), mul2(c, neg)), mul2(fma2(x.im, dx, rest.im), c)};
+    }
+  }
+  inverse_first<R1>(u, tw, lane);
+  inverse_second<R1>(u, at, lane);
+#pragma unroll
+  for (int p = 0; p < C::P; ++p)
+#pragma unroll
+    for (int m = 0; m < R1; ++m) sts(at(p, lane + 32 * m), swapped(u[p * R1 + slot<R1>(m)]));
+  fence_async_shared();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    T::store_line(&f.out, buf, ky, kb);
+    bulk_commit();
+    bulk_wait_read_all();
+  }
+}
+
 // ---- launches -----------------------------------------------------------------------------------------------
 template <class K>
 hrt_status reserve(K kernel, int bytes) {
@@ -784,11 +908,11 @@ hrt_status Passes<R1>::forward(const FftPlan& p, float* rho, bool clear, cudaStr
   using C = Cfg<R1>;
   const int kb = static_cast<int>(fft_row(C::N) / 8), smem = 4 * C::P * C::N * 16, groups = C::N * C::N / 4;
   HRT_TRY(reserve(fft_z_kernel<R1>, smem));
-  fft_z_kernel<R1><<<groups / (4 * C::P), 128, smem, s>>>(rho, p.first, p.tw, groups, 2 * static_cast<int>(fft_row(C::N)),
-                                                          clear);
+  fft_z_kernel<R1><<<groups / (4 * C::P), 128, smem, s>>>(ZForward{{rho}, {p.first}}, p.tw, groups,
+                                                          2 * static_cast<int>(fft_row(C::N)), clear);
   HRT_LAUNCHED("fft_z_kernel");
   HRT_TRY(reserve(fft_y_kernel<R1>, C::TileBytes + 1024));
-  fft_y_kernel<R1><<<C::N * kb, C::Threads, C::TileBytes + 1024, s>>>(p.y_in, p.y_out, p.tw, kb, p.err);
+  fft_y_kernel<R1><<<C::N * kb, C::Threads, C::TileBytes + 1024, s>>>(YForward{{p.y_in}, {p.y_out}}, p.tw, kb, p.err);
   HRT_LAUNCHED("fft_y_kernel");
   return HRT_OK;
 }
@@ -843,6 +967,51 @@ hrt_status Passes<R1>::inverse_z(const FftPlan& p, float* grad, float* ray, cuda
   HRT_TRY(reserve(fft_iz_kernel<R1>, smem));
   fft_iz_kernel<R1><<<dim3(groups / (4 * C::P), ray ? 5 : 3), 128, smem, s>>>(f, p.tw, groups,
                                                                              2 * static_cast<int>(fft_row(C::N)));
+  HRT_LAUNCHED("fft_iz_kernel");
+  return HRT_OK;
+}
+
+template <int R1>
+hrt_status Passes<R1>::adjoint(const FftPlan& p, double box, double pref, const FftSet& a, const float* grad_bar,
+                               float* rho_bar, cudaStream_t s) {
+  using C = Cfg<R1>;
+  const FftAdjointPlan& q = p.adjoint;
+  const int kb = static_cast<int>(fft_row(C::N) / 8), row = 2 * static_cast<int>(fft_row(C::N));
+  const int zmem = 4 * C::P * C::N * 16, groups = C::N * C::N / 4, ymem = C::TileBytes + 1024;
+  const size_t cells = static_cast<size_t>(C::N) * C::N * C::N;
+  float* g = const_cast<float*>(grad_bar);  // read only: nothing is cleared
+  HRT_TRY(reserve(fft_z_kernel<R1>, zmem));
+  HRT_TRY(reserve(fft_y_kernel<R1>, ymem));
+  // fields 0 and 1 together, then 2 through the first one's rows
+  fft_z_kernel<R1><<<dim3(groups / (4 * C::P), 2), 128, zmem, s>>>(ZForward{{g, g + cells}, {q.rows[0], q.rows[1]}}, p.tw,
+                                                                  groups, row, false);
+  HRT_LAUNCHED("fft_z_kernel");
+  fft_y_kernel<R1><<<dim3(C::N * kb, 2), C::Threads, ymem, s>>>(
+      YForward{{q.y_in[0], q.y_in[1]}, {q.y_out[0], q.y_out[1]}}, p.tw, kb, p.err);
+  HRT_LAUNCHED("fft_y_kernel");
+  fft_z_kernel<R1><<<groups / (4 * C::P), 128, zmem, s>>>(ZForward{{g + 2 * cells}, {q.rows[0]}}, p.tw, groups, row, false);
+  HRT_LAUNCHED("fft_z_kernel");
+  fft_y_kernel<R1><<<C::N * kb, C::Threads, ymem, s>>>(YForward{{q.y_in[0]}, {q.y_out[2]}}, p.tw, kb, p.err);
+  HRT_LAUNCHED("fft_y_kernel");
+  XAdjoint x{{q.x_in[0], q.x_in[1], q.x_in[2]}, q.x_out, a};
+  const auto kernel = a.g ? fft_x_adjoint_kernel<R1, true> : fft_x_adjoint_kernel<R1, false>;
+  HRT_TRY(reserve(kernel, XCfg<R1>::Bytes));
+  const float kf = static_cast<float>(2.0 * M_PI / box);
+  kernel<<<C::N * kb, C::Threads, XCfg<R1>::Bytes, s>>>(
+      x, p.tw, kb, kf, static_cast<float>(-pref / (static_cast<double>(C::N) * C::N * C::N)), p.err);
+  HRT_LAUNCHED("fft_x_adjoint_kernel");
+  YJobs y{};
+  y.jobs = 1;
+  y.in[0] = q.iy_in;
+  y.out[0] = q.iy_out;
+  HRT_TRY(reserve(fft_iy_kernel<R1>, ymem));
+  fft_iy_kernel<R1><<<C::N * kb, C::Threads, ymem, s>>>(y, p.tw, kb, kf, p.err);
+  HRT_LAUNCHED("fft_iy_kernel");
+  ZFields z{};
+  z.in[0] = q.rows[0];
+  z.out[0] = rho_bar;
+  HRT_TRY(reserve(fft_iz_kernel<R1>, zmem));
+  fft_iz_kernel<R1><<<groups / (4 * C::P), 128, zmem, s>>>(z, p.tw, groups, row);
   HRT_LAUNCHED("fft_iz_kernel");
   return HRT_OK;
 }

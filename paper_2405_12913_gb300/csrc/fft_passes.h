@@ -36,6 +36,12 @@ struct FftSet {
   float g_inv_dk;
 };
 
+// Tensor maps of the transposed solve, over the plan's five (or more) spectra: two for rows, three for tiles.
+struct FftAdjointPlan {
+  float* rows[2] = {};
+  CUtensorMap y_in[2], y_out[3], x_in[3], x_out, iy_in, iy_out;
+};
+
 // Device buffers of one mesh size and the tensor maps over them.  half holds the (y, z)-transformed density (and,
 // once the x-pass has read it, the first field of the inverse y-pass); mid the outputs of the x-pass, an x component
 // and V per filter set; out[j] field j between the inverse y- and z-passes (out[0] is half).
@@ -47,6 +53,7 @@ struct FftPlan {
   float* out[kFftMaxFields] = {};
   float* first = nullptr;  // output of the forward z-pass (mid[0])
   CUtensorMap y_in, y_out, x_in, x_out[4], iy_in[4], iy_out[kFftMaxFields];
+  FftAdjointPlan adjoint;
 };
 
 // Fills the plan's maps; half, mid[2 or 4] and out[fields] are spectra of fft_spectrum_bytes(n), 128-byte aligned.  out[0]
@@ -60,6 +67,10 @@ hrt_status launch_fft_x(const FftPlan& p, double box, double pref, const FftSet&
 // grad [3][n^3], and ray [2][n^3] (or nullptr).
 hrt_status launch_fft_inverse_y(const FftPlan& p, double box, bool rays, cudaStream_t s);
 hrt_status launch_fft_inverse_z(const FftPlan& p, float* grad, float* ray, cudaStream_t s);
+// rho_bar [n^3] from the cotangents grad_bar [3][n^3] of the fields of one filter set (hrt_pm_solve_adjoint); overwrites
+// the plan's spectra.
+hrt_status launch_fft_adjoint(const FftPlan& p, double box, double pref, const FftSet& a, const float* grad_bar, float* rho_bar,
+                              cudaStream_t s);
 // The 3D half spectrum [kx][ky][kz] (complex64) of the density last given to launch_fft_forward; half must still hold it
 // (out[0] is a buffer of its own).
 hrt_status launch_fft_spectrum(const FftPlan& p, void* out, cudaStream_t s);
@@ -71,6 +82,8 @@ struct Passes {
   static hrt_status x_pass(const FftPlan& p, double box, double pref, const FftSet& a, const FftSet* b, cudaStream_t s);
   static hrt_status inverse_y(const FftPlan& p, double box, bool rays, cudaStream_t s);
   static hrt_status inverse_z(const FftPlan& p, float* grad, float* ray, cudaStream_t s);
+  static hrt_status adjoint(const FftPlan& p, double box, double pref, const FftSet& a, const float* grad_bar, float* rho_bar,
+                            cudaStream_t s);
   static hrt_status spectrum(const FftPlan& p, void* out, cudaStream_t s);
 };
 extern template struct Passes<2>;

@@ -99,3 +99,23 @@ def test_density_spectrum_after_a_solve(hrt, n):
         pm.density_spectrum(out)
         assert (out - want).norm() <= 1e-6 * want.norm()  # log2(n^3) butterfly levels of 2^-24
         pm.close()
+
+
+@pytest.mark.parametrize("n,learned", [(64, False), (96, True), (128, False), (192, False), (256, True), (256, False), (384, False),
+                                       (512, False), (768, False)])
+def test_adjoint_matches_a_64_bit_transpose(hrt, n, learned):
+    # rho_bar = sum_j C2R(conj(H_j) R2C(g_j)) with H_j the solve's factors; the rounding bound of the solve
+    box, pref = 0.9 * n, 0.45
+    g = torch.Generator(device="cuda").manual_seed(n)
+    bar = torch.randn(3, n, n, n, device="cuda", generator=g)
+    table = (1.5 - torch.linspace(0.0, 1.0, 301, device="cuda") ** 2).float() if learned else None
+    k_max = 2.0 * math.pi * n / box / 3.0
+    f = hrt.make_filter(4.0, box / n, table, k_max) if learned else hrt.make_filter(4.0, box / n)
+    want = 0.0
+    for c in range(3):  # -d_c of the solve of each component: the transpose of an odd real operator
+        want = want - _solve64(bar[c], box, pref, 4.0, box / n, 3, table, k_max)[c]
+    pm = hrt.PM(n, box)
+    out = torch.empty(n, n, n, device="cuda")
+    pm.solve_adjoint(bar, pref, f, out)
+    assert (out - want).norm() <= 3e-6 * want.norm()
+    pm.close()
