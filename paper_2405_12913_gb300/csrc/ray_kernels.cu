@@ -648,11 +648,24 @@ hrt_status launch_rays_init(const hrt_rays& rays, const double* theta0, cudaStre
 //
 // Bound by latency and the few FP64 lanes of this part: an FP64 logarithm and square root and three FP64 shared-memory
 // atomics per mode, most lanes of a warp on the same bin, took 880 us at m = 2048.  A warp now takes 256 columns of
-// the rows nx and -nx, whose geometry is the same; a lane's modes climb through the bins, so it adds in registers and
-// goes to shared memory when its bin changes (rarely) and, after a sum over the warp, at the end.  |n| is a float
-// square root with its residual (2^-46); the power is summed in FP64.
+// the rows nx and -nx, whose geometry is the same; a lane's modes climb through the bins, so it adds in registers, and
+// what lanes hold goes to shared memory, summed over the warp, where a bin ends and at the end: 70 us with a shared-memory
+// atomic per lane there, 34 us with the sum.  |n| is a float
+// square root with its residual (2^-46), squares are float pairs and partial sums become FP64 when they leave the lane.
 // ---------------------------------------------------------------------------------------------------------
 constexpr int kBinColumns = 256;
+
+// Whether x^2, its rounding error and sums of a warp's many stay within float's normal range (0 does; NaN does not).
+__device__ __forceinline__ bool moderate(float x) { return x == 0.f || (fabsf(x) > 1e-12f && fabsf(x) < 1e15f); }
+__device__ __forceinline__ bool moderate(float2 z) { return moderate(z.x) && moderate(z.y); }
+
+// hi + lo += scale x^2 with the rounding errors kept; scale a power of two.
+__device__ __forceinline__ void add_square(float x, float scale, float& hi, float& lo) {
+  const float sx = scale * x, q = __fmul_rn(sx, x), e = __fmaf_rn(sx, x, -q);
+  const float sum = __fadd_rn(hi, q), back = __fsub_rn(sum, hi);
+  lo += __fadd_rn(__fsub_rn(hi, __fsub_rn(sum, back)), __fsub_rn(q, back)) + e;
+  hi = sum;
+}
 
 __global__ void __launch_bounds__(256) power_bin_kernel(const float2* __restrict__ spec, int m, double ell_scale,
                                                         double p_norm, int nbins,
@@ -692,63 +705,84 @@ __global__ void __launch_bounds__(256) power_bin_kernel(const float2* __restrict
         }
       }
     }
+    // squares as float pairs (2^-48) where no square or its rounding error can leave float's range, else in FP64
+    bool small = true;
+#pragma unroll
+    for (int i = 0; i < kBinColumns / 32; ++i) small = small && moderate(u[i]) && moderate(v[i]);
+    const bool plain = __all_sync(0xffffffffu, small);
     double power = 0.0;
-    float ell_hi = 0.f, ell_lo = 0.f;
+    float pw_hi = 0.f, pw_lo = 0.f, ell_hi = 0.f, ell_lo = 0.f;
     int count = 0;
-    auto flush = [&] {
-      if (count > 0 && bin >= 0 && bin < nbins) {
-        atomicAdd(sh + bin, power * p_norm);
-        atomicAdd(sh + nbins + bin, (static_cast<double>(ell_hi) + ell_lo) * ell_scale);
-        atomicAdd(sh + 2 * nbins + bin, static_cast<double>(count));
+    // what the lanes with `out` hold of their bins, summed over the lanes of the same bin; by the whole warp
+    auto drain = [&](bool out) {
+      const double ell = (static_cast<double>(ell_hi) + ell_lo) * ell_scale;
+      const double all = (power + (static_cast<double>(pw_hi) + pw_lo)) * p_norm;
+      unsigned left = __ballot_sync(0xffffffffu, out && count > 0 && bin >= 0 && bin < nbins);
+      while (left) {
+        const int leader = __ffs(left) - 1;
+        const int leading = __shfl_sync(0xffffffffu, bin, leader);  // by every lane: not behind a short circuit
+        const bool mine = ((left >> lane) & 1u) && bin == leading;
+        double p = mine ? all : 0.0, e = mine ? ell : 0.0;
+        int c = mine ? count : 0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          p += __shfl_xor_sync(0xffffffffu, p, o);
+          e += __shfl_xor_sync(0xffffffffu, e, o);
+          c += __shfl_xor_sync(0xffffffffu, c, o);
+        }
+        if (lane == leader) {
+          atomicAdd(sh + bin, p);
+          atomicAdd(sh + nbins + bin, e);
+          atomicAdd(sh + 2 * nbins + bin, static_cast<double>(c));
+        }
+        left &= ~__ballot_sync(0xffffffffu, mine);
       }
-      power = 0.0;
-      ell_hi = ell_lo = 0.f;
-      count = 0;
+      if (out) {
+        power = 0.0;
+        pw_hi = pw_lo = ell_hi = ell_lo = 0.f;
+        count = 0;
+      }
     };
 #pragma unroll
     for (int i = 0; i < kBinColumns / 32; ++i) {
       const int iz = z0 + 32 * i;
       const int n2 = nx * nx + iz * iz;
-      if (iz >= mzc || n2 == 0) continue;
-      if (bin < nbins && n2 >= edge[bin + 1]) {
-        flush();
-        do ++bin;
-        while (bin < nbins && n2 >= edge[bin + 1]);
+      const bool mode = iz < mzc && n2 > 0;
+      const bool next = mode && bin < nbins && n2 >= edge[bin + 1];
+      if (__any_sync(0xffffffffu, next)) {
+        drain(next);
+        if (next) {
+          do ++bin;
+          while (bin < nbins && n2 >= edge[bin + 1]);
+        }
+        __syncwarp();
       }
-      const int each = iz == 0 || iz == m / 2 ? 1 : 2, modes = two ? 2 * each : each;
-      double pw = static_cast<double>(u[i].x) * u[i].x + static_cast<double>(u[i].y) * u[i].y;
-      if (two) pw += static_cast<double>(v[i].x) * v[i].x + static_cast<double>(v[i].y) * v[i].y;
-      power += each == 2 ? 2.0 * pw : pw;
-      count += modes;
-      // modes |n| as hi + lo, added with the rounding error kept (modes is a power of two)
-      const float a = static_cast<float>(n2), rest = static_cast<float>(n2 - static_cast<int>(a));
-      const float s = sqrtf(a), corr = (__fmaf_rn(-s, s, a) + rest) / (2.f * s);
-      const float x = s * modes, sum = ell_hi + x, back = sum - ell_hi;
-      ell_lo += ((ell_hi - (sum - back)) + (x - back)) + corr * modes;
-      ell_hi = sum;
+      if (mode) {
+        const int each = iz == 0 || iz == m / 2 ? 1 : 2, modes = two ? 2 * each : each;
+        const float scale = static_cast<float>(each);
+        if (plain) {
+          add_square(u[i].x, scale, pw_hi, pw_lo);
+          add_square(u[i].y, scale, pw_hi, pw_lo);
+          if (two) {
+            add_square(v[i].x, scale, pw_hi, pw_lo);
+            add_square(v[i].y, scale, pw_hi, pw_lo);
+          }
+        } else {
+          double pw = static_cast<double>(u[i].x) * u[i].x + static_cast<double>(u[i].y) * u[i].y;
+          if (two) pw += static_cast<double>(v[i].x) * v[i].x + static_cast<double>(v[i].y) * v[i].y;
+          power += each == 2 ? 2.0 * pw : pw;
+        }
+        count += modes;
+        // modes |n| as hi + lo, added with the rounding error kept (modes is a power of two)
+        const float a = static_cast<float>(n2), rest = static_cast<float>(n2 - static_cast<int>(a));
+        const float s = sqrtf(a), corr = (__fmaf_rn(-s, s, a) + rest) / (2.f * s);
+        const float x = s * modes, sum = ell_hi + x, back = sum - ell_hi;
+        ell_lo += ((ell_hi - (sum - back)) + (x - back)) + corr * modes;
+        ell_hi = sum;
+      }
+      __syncwarp();
     }
-    // what is left of each bin, summed over the warp's lanes that hold it
-    unsigned left = __ballot_sync(0xffffffffu, count > 0 && bin >= 0 && bin < nbins);
-    const double ell = (static_cast<double>(ell_hi) + ell_lo) * ell_scale;
-    while (left) {
-      const int leader = __ffs(left) - 1;
-      const int leading = __shfl_sync(0xffffffffu, bin, leader);  // by every lane: not behind a short circuit
-      const bool mine = ((left >> lane) & 1u) && bin == leading;
-      double p = mine ? power * p_norm : 0.0, e = mine ? ell : 0.0;
-      int c = mine ? count : 0;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        p += __shfl_xor_sync(0xffffffffu, p, o);
-        e += __shfl_xor_sync(0xffffffffu, e, o);
-        c += __shfl_xor_sync(0xffffffffu, c, o);
-      }
-      if (lane == leader) {
-        atomicAdd(sh + bin, p);
-        atomicAdd(sh + nbins + bin, e);
-        atomicAdd(sh + 2 * nbins + bin, static_cast<double>(c));
-      }
-      left &= ~__ballot_sync(0xffffffffu, mine);
-    }
+    drain(true);
   }
   __syncthreads();
   for (int i = threadIdx.x; i < 3 * nbins; i += blockDim.x)
