@@ -298,8 +298,8 @@ struct hrt_pm {
   double box = 0.0;
   int32_t n_ray = 0;
   cudaStream_t stream = nullptr;
-  cufftHandle r2c = 0, c2r = 0;
-  bool have_r2c = false, have_c2r = false;
+  cufftHandle r2c = 0, c2r = 0, c2r3 = 0;  // c2r3: the three particle fields in one batch (small sides of the 3D path)
+  bool have_r2c = false, have_c2r = false, have_c2r3 = false;
   void* work = nullptr;
   void* rho_hat = nullptr;
   void* grad_hat = nullptr;     // 3 + n_ray spectra
@@ -355,6 +355,10 @@ static void pm_set_work(hrt_pm* pm) {
     cufftSetWorkArea(p, pm->work);
     cufftSetStream(p, pm->stream);
   }
+  if (pm->have_c2r3) {
+    cufftSetWorkArea(pm->c2r3, pm->work);
+    cufftSetStream(pm->c2r3, pm->stream);
+  }
   if (pm->have_cb3) {
     cufftSetWorkArea(pm->c2r_cb3, pm->work);
     cufftSetStream(pm->c2r_cb3, pm->stream);
@@ -392,6 +396,11 @@ static hrt_status pm_make_split(hrt_pm* pm) {
   return HRT_OK;
 }
 
+// Largest side of the 3D path whose three inverse transforms go as one batch: at small sides the launches count (three of 4
+// to 5 us per transform).  A solve, three transforms and one batch: 60^3 56 and 38 us, 100^3 83 and 54, 144^3 116 and 92,
+// 240^3 536 and 526, 300^3 971 and 1035.
+constexpr int64_t kBatchSide = 240;
+
 static hrt_status pm_make(int64_t n, double box, int32_t n_ray, cudaStream_t s, hrt_pm* pm) {
   pm->n = n;
   pm->box = box;
@@ -408,6 +417,13 @@ static hrt_status pm_make(int64_t n, double box, int32_t n_ray, cudaStream_t s, 
   HRT_CUFFT(cufftSetAutoAllocation(pm->c2r, 0));
   HRT_CUFFT(cufftMakePlanMany64(pm->c2r, 3, dims, nullptr, 1, 0, nullptr, 1, 0, CUFFT_C2R, 1, &w2));
   pm->work_bytes = std::max(w1, w2);
+  if (!fft_supported(n) && n <= kBatchSide) {
+    HRT_CUFFT(cufftCreate(&pm->c2r3));
+    pm->have_c2r3 = true;
+    HRT_CUFFT(cufftSetAutoAllocation(pm->c2r3, 0));
+    HRT_CUFFT(cufftMakePlanMany64(pm->c2r3, 3, dims, nullptr, 1, 0, nullptr, 1, 0, CUFFT_C2R, 3, &w1));
+    pm->work_bytes = std::max(pm->work_bytes, w1);
+  }
   HRT_TRY(device_alloc(&pm->work, pm->work_bytes, s, "cuFFT work area"));
   pm_set_work(pm);
   HRT_TRY(device_alloc(&pm->rho_hat, spectrum_alloc(n), s, "rho_hat"));
@@ -451,6 +467,7 @@ static void pm_release(hrt_pm* pm) {
   cudaStreamSynchronize(pm->stream);
   if (pm->have_r2c) cufftDestroy(pm->r2c);
   if (pm->have_c2r) cufftDestroy(pm->c2r);
+  if (pm->have_c2r3) cufftDestroy(pm->c2r3);
   if (pm->have_cb3) cufftDestroy(pm->c2r_cb3);
   if (pm->have_cb2) cufftDestroy(pm->c2r_cb2);
   device_free(pm->twiddles, pm->stream);
@@ -562,8 +579,11 @@ static hrt_status pm_solve(hrt_pm* pm, float* rho, double pref, const hrt_filter
   }
   if (before_fields) HRT_CUDA(cudaStreamWaitEvent(pm->stream, before_fields, 0));
   PhaseScope ps(pc, 5);
-  for (int j = 0; j < 3; ++j)
-    HRT_CUFFT(cufftExecC2R(pm->c2r, reinterpret_cast<cufftComplex*>(gh + j * sb), grad + j * mb));
+  if (pm->have_c2r3)
+    HRT_CUFFT(cufftExecC2R(pm->c2r3, reinterpret_cast<cufftComplex*>(gh), grad));
+  else
+    for (int j = 0; j < 3; ++j)
+      HRT_CUFFT(cufftExecC2R(pm->c2r, reinterpret_cast<cufftComplex*>(gh + j * sb), grad + j * mb));
   if (rays)
     for (int j = 0; j < pm->n_ray; ++j)
       HRT_CUFFT(cufftExecC2R(pm->c2r, reinterpret_cast<cufftComplex*>(gh + (3 + j) * sb), ray_grad + j * mb));
