@@ -352,13 +352,55 @@ __device__ void half_forward(const RayStepParams& p, int j0, int j1, double thx,
   }
 }
 
+// Sums of a, b and c over the warp in lanes 0, 8 and 16: the lanes of a half first exchange what the other half will
+// finish, seven shuffles in all where three separate sums take fifteen.
+__device__ __forceinline__ float warp_sum3(float a, float b, float c, int lane) {
+  const unsigned full = 0xffffffffu;
+  // lanes 0..15 go on with a and b, lanes 16..31 with c
+  const float a2 = __shfl_xor_sync(full, a, 16), b2 = __shfl_xor_sync(full, b, 16), c2 = __shfl_xor_sync(full, c, 16);
+  const bool upper = (lane & 16) != 0;
+  a += a2;
+  b += b2;
+  c += c2;
+  // of those, lanes with bit 3 go on with b
+  const float give = upper ? c : (lane & 8) ? a : b, keep = upper ? c : (lane & 8) ? b : a;
+  float v = keep + __shfl_xor_sync(full, give, 8);
+  v += __shfl_xor_sync(full, v, 4);
+  v += __shfl_xor_sync(full, v, 2);
+  v += __shfl_xor_sync(full, v, 1);
+  return v;
+}
+
+// f[iz] += (1 - fz) q, f[jz] += fz q on a mesh column f; wide: the column starts on a 16-byte boundary (n a multiple of 4).
+// One reduction of the aligned four cells carries both unless jz starts the next four (iz mod 4 = 3, the wrap included).
+__device__ __forceinline__ void column_add(float* __restrict__ f, int iz, int jz, float fz, float q, bool wide) {
+  if (q == 0.f) return;
+  const float lo = (1.f - fz) * q, hi = fz * q;
+  const int s = iz & 3;
+  if (wide && s < 3) {
+    atomicAdd(reinterpret_cast<float4*>(f + (iz - s)), make_float4(s == 0 ? lo : 0.f, s == 1 ? lo : s == 0 ? hi : 0.f,
+                                                                   s == 2 ? lo : s == 1 ? hi : 0.f, s == 2 ? hi : 0.f));
+    return;
+  }
+  if (lo != 0.f) atomicAdd(f + iz, lo);
+  if (hi != 0.f) atomicAdd(f + jz, hi);
+}
+
 // Backward of one half kick: given Kbar, Jbar, accumulate theta_bar (FP64-free float32), field cotangents and the
 // node-coefficient cotangents (per block, in shared memory: [3][n_nodes] = cw_bar, cwr_bar, chi_bar).
+//
+// Bound by instruction issue.  Neighbouring rays of a warp mostly share the node's mesh cell: lanes with the same cell that
+// follow each other form a segment, a segmented shuffle reduction sums its cotangents and its first lane issues the
+// atomics (a cell that reappears later in the warp starts a new segment).  All rays have a node's z in common, so that
+// the eight corner sums before the split over the two z planes are reduced, in as many rounds as the warp's
+// longest segment needs, and the two rows of a 16 x 2 warp meet where both have a segment of the cell on the same
+// column.
 __device__ void half_backward(const RayStepParams& p, int j0, int j1, double thx, double thy, double ref_r,
                               const float* __restrict__ gx, const float* __restrict__ gy, const float Kb[2],
                               const float Jb[2][2], float* __restrict__ gbx, float* __restrict__ gby, float thb[2],
-                              float* __restrict__ sh_nodes, int n_nodes, bool active) {
+                              float* __restrict__ sh_nodes, int n_nodes, bool active, bool wide) {
   if (j1 <= j0) return;
+  const unsigned full = 0xffffffffu;
   int bx = 0, by = 0;
   float fbx = 0.f, fby = 0.f;
   if (active) {
@@ -366,14 +408,14 @@ __device__ void half_backward(const RayStepParams& p, int j0, int j1, double thx
     base_pos(p, p.obs_y, ref_r, thy, by, fby);
   }
   const float tx = static_cast<float>(thx), ty = static_cast<float>(thy);
-  const float inv_cell = static_cast<float>(1.0 / p.cell);
+  const float inv_cell = static_cast<float>(1.0 / p.cell), ref_cells = static_cast<float>(ref_r / p.cell);
   const float* f[2] = {gx, gy};
   float* fb[2] = {gbx, gby};
   const int lane = threadIdx.x & 31;
   for (int j = j0; j < j1; ++j) {
     float cwb = 0.f, cwrb = 0.f, chib = 0.f;
     NodeCols c{};
-    float t[2][4][2] = {};  // field cotangent per field, (x, y) corner and z plane
+    float q[2][4] = {};  // field cotangent per field and (x, y) corner, over both z planes
     if (active) {
       node_cols(p, j, bx, fbx, by, fby, tx, ty, c);
       const float cw = p.cw[j], cwr = p.cwr[j];
@@ -383,15 +425,12 @@ __device__ void half_backward(const RayStepParams& p, int j0, int j1, double thx
         const NodeField o = node_field(f[a], c);
         // K_a = cw v_a and J_ab = cwr d_b v_a (b = x, y): cotangent weights of v, dx v, dy v
         const float al = cw * Kb[a], bex = cwr * Jb[a][0], bey = cwr * Jb[a][1];
-        // field cotangents: w_k = WX WY WZ, d w_k / d fx = SX WY WZ, ... -> per (x, y) corner, times WZ
+        // field cotangents: w_k = WX WY WZ, d w_k / d fx = SX WY WZ, ... -> per (x, y) corner, without WZ
         const float ux = 1.f - c.fx, uy = 1.f - c.fy;
-        const float q[4] = {al * ux * uy - bex * uy - bey * ux, al * ux * c.fy - bex * c.fy + bey * ux,
-                            al * c.fx * uy + bex * uy - bey * c.fx, al * c.fx * c.fy + bex * c.fy + bey * c.fx};
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          t[a][k][0] = (1.f - c.fz) * q[k];
-          t[a][k][1] = c.fz * q[k];
-        }
+        q[a][0] = al * ux * uy - bex * uy - bey * ux;
+        q[a][1] = al * ux * c.fy - bex * c.fy + bey * ux;
+        q[a][2] = al * c.fx * uy + bex * uy - bey * c.fx;
+        q[a][3] = al * c.fx * c.fy + bex * c.fy + bey * c.fx;
         // cotangent of the fractional position (the mixed second derivatives couple the J terms)
         fbar_x += al * o.dx + bey * o.sxy;
         fbar_y += al * o.dy + bex * o.sxy;
@@ -400,51 +439,51 @@ __device__ void half_backward(const RayStepParams& p, int j0, int j1, double thx
         cwrb += Jb[a][0] * o.dx + Jb[a][1] * o.dy;
       }
       // f_x = (O_x + chi_j theta_x) / cell - cell index: d f_x / d theta_x = chi_j / cell, d f / d chi_j = theta/cell
-      const float r_over_cell = static_cast<float>(ref_r / p.cell) + p.dr[j];
+      const float r_over_cell = ref_cells + p.dr[j];
       thb[0] += fbar_x * r_over_cell;
       thb[1] += fbar_y * r_over_cell;
       chib = (fbar_x * tx + fbar_y * ty + fbar_z) * inv_cell;
     }
-    // Neighbouring rays of a warp mostly share the node's mesh cell: lanes with the same cell that follow
-    // each other form a segment, the segment's cotangents are summed by a segmented shuffle reduction and its
-    // first lane issues the 16 atomics (a cell that reappears later in the warp starts a new segment).
-    const long long key = active ? static_cast<long long>(c.r[0] + c.iz) : -1ll - lane;
-    const long long prev = __shfl_up_sync(0xffffffffu, key, 1);
-    const bool head = lane == 0 || prev != key;
-    const unsigned heads = __ballot_sync(0xffffffffu, head);
-    const unsigned above = lane == 31 ? 0u : heads & (0xffffffffu << (lane + 1));
+    // segments of equal columns (z is the same), broken between the two rows of a warp
+    const long long key = active ? static_cast<long long>(c.r[0]) : -1ll - lane;
+    const long long prev = __shfl_up_sync(full, key, 1);
+    const bool head = (lane & 15) == 0 || prev != key;
+    const unsigned heads = __ballot_sync(full, head);
+    const unsigned above = lane == 31 ? 0u : heads & (full << (lane + 1));
     const int seg_end = above ? __ffs(above) - 2 : 31;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1)
-#pragma unroll
-      for (int a = 0; a < 2; ++a)
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-#pragma unroll
-          for (int z = 0; z < 2; ++z) {
-            const float u = __shfl_down_sync(0xffffffffu, t[a][k][z], d);
-            if (lane + d <= seg_end) t[a][k][z] += u;
-          }
-    if (head && active) {
+    for (int d = 1; d < 16; d <<= 1) {
+      const bool more = lane + d <= seg_end;
+      if (!__any_sync(full, more)) break;  // no segment is longer than d
 #pragma unroll
       for (int a = 0; a < 2; ++a)
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-          if (t[a][k][0] != 0.f) atomicAdd(fb[a] + c.r[k] + c.iz, t[a][k][0]);
-          if (t[a][k][1] != 0.f) atomicAdd(fb[a] + c.r[k] + c.jz, t[a][k][1]);
+          const float u = __shfl_down_sync(full, q[a][k], d);
+          if (more) q[a][k] += u;
         }
     }
+    // a head of the upper row joins the head of the lower row 16 lanes below, where the columns are the same
+    const long long other = __shfl_xor_sync(full, key, 16);
+    const bool join = head && ((heads >> (lane ^ 16)) & 1u) && other == key;
+    if (__any_sync(full, join)) {
+#pragma unroll
+      for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const float u = __shfl_down_sync(full, q[a][k], 16);
+          if (join && lane < 16) q[a][k] += u;
+        }
+    }
+    if (head && active && !(join && lane >= 16)) {
+      const float fz = p.fz[j];
+#pragma unroll
+      for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) column_add(fb[a] + c.r[k], c.iz, c.jz, fz, q[a][k], wide);
+    }
     // block reduction of the node cotangents into shared memory
-    for (int o = 16; o > 0; o >>= 1) {
-      cwb += __shfl_down_sync(0xffffffffu, cwb, o);
-      cwrb += __shfl_down_sync(0xffffffffu, cwrb, o);
-      chib += __shfl_down_sync(0xffffffffu, chib, o);
-    }
-    if ((threadIdx.x & 31) == 0) {
-      atomicAdd(sh_nodes + j, cwb);
-      atomicAdd(sh_nodes + n_nodes + j, cwrb);
-      atomicAdd(sh_nodes + 2 * n_nodes + j, chib);
-    }
+    const float sum = warp_sum3(cwb, cwrb, chib, lane);
+    if ((lane & 7) == 0 && lane < 24) atomicAdd(sh_nodes + (lane >> 3) * n_nodes + j, sum);
   }
 }
 
@@ -664,6 +703,8 @@ __global__ void __launch_bounds__(128) ray_step_adjoint_kernel(
     r = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   }
   const bool active = r < nr;
+  // 16-byte reductions into the field cotangents
+  const bool wide = (p.n & 3) == 0 && ((reinterpret_cast<uintptr_t>(gbx) | reinterpret_cast<uintptr_t>(gby)) & 15) == 0;
   double db = 0.0;
   double2 th0 = active ? theta[r] : make_double2(0.0, 0.0);
   const float2 et0 = active ? eta[r] : make_float2(0.f, 0.f);
@@ -713,7 +754,7 @@ __global__ void __launch_bounds__(128) ray_step_adjoint_kernel(
     half_backward_tiled(p, p.n1, p.n1 + p.n2, th1x, th1y, p.ref_r[1], gx, gy, gz, Kb, Jb, gbx, gby, gbz, thb1, sh,
                         n_nodes, active);
   else
-    half_backward(p, p.n1, p.n1 + p.n2, th1x, th1y, p.ref_r[1], gx, gy, Kb, Jb, gbx, gby, thb1, sh, n_nodes, active);
+    half_backward(p, p.n1, p.n1 + p.n2, th1x, th1y, p.ref_r[1], gx, gy, Kb, Jb, gbx, gby, thb1, sh, n_nodes, active, wide);
   // A1 = A0 + d B1
   for (int a = 0; a < 2; ++a)
     for (int b = 0; b < 2; ++b) {
@@ -737,7 +778,7 @@ __global__ void __launch_bounds__(128) ray_step_adjoint_kernel(
     half_backward_tiled(p, 0, p.n1, th0.x, th0.y, p.ref_r[0], gx, gy, gz, Kb, Jb, gbx, gby, gbz, thb0, sh, n_nodes,
                         active);
   else
-    half_backward(p, 0, p.n1, th0.x, th0.y, p.ref_r[0], gx, gy, Kb, Jb, gbx, gby, thb0, sh, n_nodes, active);
+    half_backward(p, 0, p.n1, th0.x, th0.y, p.ref_r[0], gx, gy, Kb, Jb, gbx, gby, thb0, sh, n_nodes, active, wide);
   if (active) {
     theta_bar[r] = make_double2(thb0[0], thb0[1]);
     eta_bar[r] = make_float2(etb[0], etb[1]);
