@@ -317,7 +317,7 @@ struct hrt_pm {
   bool split = false;
   hrt::FftPlan fft;
   float2* twiddles = nullptr;
-  void* split_hat = nullptr;
+  void* split_hat = nullptr;  // work, until the callback plans need a larger one
   int* xerr = nullptr;      // device error word of the kernels that wait for TMA copies (FFT passes, tiled deposit)
   bool last_split = false;  // the last solve took the split path: rho_hat holds no 3D spectrum
 };
@@ -372,7 +372,7 @@ static void pm_set_work(hrt_pm* pm) {
 // Buffers, twiddles and tensor maps of the FFT passes.
 static hrt_status pm_make_split(hrt_pm* pm) {
   const size_t sp = spectrum_alloc(pm->n);
-  HRT_TRY(device_alloc(&pm->split_hat, sp * split_spectra(pm->n, pm->n_ray), pm->stream, "spectra of the FFT passes"));
+  pm->split_hat = pm->work;
   std::vector<float2> tw;
   fft_twiddles(pm->n, tw);
   HRT_TRY(device_alloc(reinterpret_cast<void**>(&pm->xerr), sizeof(int), pm->stream, "FFT pass error word"));
@@ -424,6 +424,9 @@ static hrt_status pm_make(int64_t n, double box, int32_t n_ray, cudaStream_t s, 
     HRT_CUFFT(cufftMakePlanMany64(pm->c2r3, 3, dims, nullptr, 1, 0, nullptr, 1, 0, CUFFT_C2R, 3, &w1));
     pm->work_bytes = std::max(pm->work_bytes, w1);
   }
+  // The spectra that the FFT passes need on top lie in the cuFFT work area: the plans and the passes take turns on one
+  // stream, and neither expects to find there what it left.
+  if (fft_supported(n)) pm->work_bytes = std::max(pm->work_bytes, spectrum_alloc(n) * split_spectra(n, n_ray));
   HRT_TRY(device_alloc(&pm->work, pm->work_bytes, s, "cuFFT work area"));
   pm_set_work(pm);
   HRT_TRY(device_alloc(&pm->rho_hat, spectrum_alloc(n), s, "rho_hat"));
@@ -453,7 +456,7 @@ static hrt_status pm_build_fused(hrt_pm* pm) {
   }
   const size_t need = std::max(w3, w4);
   if (need > pm->work_bytes) {
-    device_free(pm->work, pm->stream);
+    if (pm->split_hat != pm->work) device_free(pm->work, pm->stream);  // else it stays with the FFT passes
     pm->work = nullptr;
     HRT_TRY(device_alloc(&pm->work, need, pm->stream, "cuFFT work area"));
     pm->work_bytes = need;
@@ -471,7 +474,7 @@ static void pm_release(hrt_pm* pm) {
   if (pm->have_cb3) cufftDestroy(pm->c2r_cb3);
   if (pm->have_cb2) cufftDestroy(pm->c2r_cb2);
   device_free(pm->twiddles, pm->stream);
-  device_free(pm->split_hat, pm->stream);
+  if (pm->split_hat != pm->work) device_free(pm->split_hat, pm->stream);
   device_free(pm->xerr, pm->stream);
   device_free(pm->work, pm->stream);
   device_free(pm->rho_hat, pm->stream);
@@ -1713,8 +1716,10 @@ hrt_status hrt_workspace_bytes(const hrt_config* cfg, int64_t n_rays, size_t* by
   if (!bytes || n_rays < 0) return fail(HRT_ERR_INVALID_ARG, "bad arguments");
   const size_t n = cfg->n_mesh, mesh = n * n * n * sizeof(float), np = cfg->n_side * cfg->n_side * cfg->n_side;
   size_t b = 6 * np * sizeof(float) + mesh * (4 + cfg->ray_fields);
-  b += spectrum_alloc(cfg->n_mesh) * (1 + 3 + cfg->ray_fields) + 2 * spectrum_bytes(cfg->n_mesh);  // + cuFFT work
-  if (fft_supported(cfg->n_mesh)) b += fft_spectrum_bytes(cfg->n_mesh) * split_spectra(cfg->n_mesh, cfg->ray_fields);
+  size_t work = 2 * spectrum_bytes(cfg->n_mesh);  // cuFFT, and the further spectra of the FFT passes in its place
+  if (fft_supported(cfg->n_mesh))
+    work = std::max(work, fft_spectrum_bytes(cfg->n_mesh) * split_spectra(cfg->n_mesh, cfg->ray_fields));
+  b += spectrum_alloc(cfg->n_mesh) * (1 + 3 + cfg->ray_fields) + work;
   b += static_cast<size_t>(n_rays) * (2 * sizeof(double) + 10 * sizeof(float));
   b += static_cast<size_t>(n_rays) * 4 * sizeof(float) * cfg->n_sources;
   // cell-order storage of the particles (on by default): second copies, two order maps, keys, ranks, sources and
