@@ -121,7 +121,10 @@ struct RayStepParams {
 // gz (the third gradient component) is read only when p.tiled.
 hrt_status launch_ray_step(const hrt_rays& rays, const float* gx, const float* gy, const RayStepParams& p,
                            float* maps, cudaStream_t s, const float* gz = nullptr);
-// Gives back the idle workspace of launch_ray_step on the current device.
+// Workspace for planes copied out of the mesh, stream-ordered (cudaFreeAsync on s gives it back to its pool); nullptr if there
+// is none to be had or the stream is being captured.
+void* plane_workspace(size_t bytes, cudaStream_t s);
+// Gives back the idle workspace of plane_workspace on the current device.
 void ray_planes_release();
 hrt_status launch_ray_drift_free(const hrt_rays& rays, double d, cudaStream_t s);
 hrt_status launch_ray_readout(const hrt_rays& rays, float* maps, cudaStream_t s);

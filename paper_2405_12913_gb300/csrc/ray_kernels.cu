@@ -492,7 +492,7 @@ __global__ void __launch_bounds__(128, G == Gather::kPlanes ? 4 : 1) ray_step_ke
   }
 }
 
-// Workspace of the node planes: stream-ordered from a pool of the library's own, which keeps at most kPlanePoolBytes per
+// Workspace of planes: stream-ordered from a pool of the library's own, which keeps at most kPlanePoolBytes per
 // device between calls (given back by ray_planes_release).
 constexpr size_t kPlaneBytes = size_t{96} << 20, kPlanePoolBytes = size_t{128} << 20;
 constexpr int kPoolDevices = 16;
@@ -527,6 +527,19 @@ void ray_planes_release() {
   if (g_plane_pool[dev]) cudaMemPoolTrimTo(g_plane_pool[dev], 0);
 }
 
+void* plane_workspace(size_t bytes, cudaStream_t s) {
+  cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &capturing) != cudaSuccess || capturing != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  cudaMemPool_t pool = plane_pool();
+  void* work = nullptr;
+  if (pool && cudaMallocFromPoolAsync(&work, bytes, pool, s) == cudaSuccess) return work;
+  cudaGetLastError();
+  return nullptr;
+}
+
 // Rays times nodes from which the three small launches before the step's pay (the gather does about 150 per ns).
 constexpr int64_t kPlaneRays = 1 << 14, kPlaneWork = 1 << 22;
 
@@ -538,14 +551,12 @@ hrt_status launch_ray_step(const hrt_rays& rays, const float* gx, const float* g
   RayPlanes q{};
   const int nodes = p.n1 + p.n2;
   char* work = nullptr;
-  cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
-  if (!p.tiled && !p.theta32 && rays.n_rays >= kPlaneRays && rays.n_rays * nodes >= kPlaneWork &&
-      cudaStreamIsCapturing(s, &capturing) == cudaSuccess && capturing == cudaStreamCaptureStatusNone) {
-    // a step without the workspace (or being captured) gathers from the fields
+  if (!p.tiled && !p.theta32 && rays.n_rays >= kPlaneRays && rays.n_rays * nodes >= kPlaneWork) {
+    // a step without the workspace gathers from the fields
     const size_t most = static_cast<size_t>(nodes) * rays.n_rays * sizeof(float2);  // no more cells than rays
     const size_t bytes = most < kPlaneBytes ? most : kPlaneBytes;
-    cudaMemPool_t pool = plane_pool();
-    if (pool && cudaMallocFromPoolAsync(reinterpret_cast<void**>(&work), 256 + bytes, pool, s) == cudaSuccess) {
+    work = static_cast<char*>(plane_workspace(256 + bytes, s));
+    if (work) {
       q.key = reinterpret_cast<unsigned long long*>(work);
       q.done = reinterpret_cast<unsigned*>(work + 32);
       q.box = reinterpret_cast<PlaneBox*>(work + 48);
@@ -554,9 +565,6 @@ hrt_status launch_ray_step(const hrt_rays& rays, const float* gx, const float* g
       q.r_lo = p.r_lo;
       q.r_hi = p.r_hi;
       kernel = ray_step_kernel<Gather::kPlanes>;
-    } else {
-      cudaGetLastError();
-      work = nullptr;
     }
   }
   if (work) {

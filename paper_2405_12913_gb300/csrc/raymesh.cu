@@ -79,6 +79,133 @@ __device__ __forceinline__ int wrap(int i, int n) {
 // Box index along the box axis that receives a sky axis: i -> sgn i + sh (mod n).
 __device__ __forceinline__ int box_index(int i, int sgn, int sh, int n) { return wrap(sgn > 0 ? i + sh : sh - i, n); }
 
+// Planes of the 3D mesh, copied for the projection: (d_x phi, d_y phi) of every plane of the half shell over the cells
+// x0 .. x0 + ex - 1, y0 .. y0 + ey - 1 (unwrapped) as [plane][x][y].  A warp of the projection has 32 neighbouring y, whose
+// columns lie a mesh row apart in the fields: there each of its two loads per plane touches 15 sectors, here one load
+// touches two or three.  A 512^3 mesh and 1024^2 ray-mesh nodes, 27 planes: copy 29 and projection 84 us against 172 us
+// from the fields; with the general kernel's loops the planes alone gained nothing (140 us and the copy).
+struct PlaneSlab {
+  float2* data;
+  int x0, y0, ex, ey;
+  int row0;  // first ray-mesh row of the slab
+};
+// Bytes of a slab: the planes stay in L2 between the copy and the projection; a larger mesh goes in slabs of rows.
+constexpr int64_t kSlabBytes = int64_t{60} << 20;
+// Ray-mesh nodes times planes from which a second launch per half shell pays.
+constexpr int64_t kSlabWork = 1 << 20;
+
+// A block copies 32 planes of 8 x 8 cells: a lane per plane, so that a warp reads a column's run of z as it lies, and rows of
+// y leave through shared memory.
+constexpr int kCopyPlanes = 32, kCopySide = 8;
+
+__global__ void __launch_bounds__(256) raymesh_planes_kernel(const float* __restrict__ gx, const float* __restrict__ gy,
+                                                             const __grid_constant__ ProjectParams p, PlaneSlab v) {
+  __shared__ float2 tile[kCopySide * kCopySide][kCopyPlanes + 1];
+  const int n = p.n, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int chunks = (p.n_planes + kCopyPlanes - 1) / kCopyPlanes, tiles_y = (v.ey + kCopySide - 1) / kCopySide;
+  const int t = blockIdx.x / chunks, q0 = (blockIdx.x - t * chunks) * kCopyPlanes, tx = t / tiles_y;
+  const int x0 = tx * kCopySide, y0 = (t - tx * tiles_y) * kCopySide;
+  const int iz = p.kz[min(q0 + lane, p.n_planes - 1)];
+  const int64_t row = static_cast<int64_t>(wrap(v.x0 + x0 + warp, n)) * n;
+  float ax[kCopySide], ay[kCopySide];
+#pragma unroll
+  for (int y = 0; y < kCopySide; ++y) {  // cells past the slab: read, not written
+    const int64_t at = (row + wrap(v.y0 + y0 + y, n)) * n + iz;
+    ax[y] = __ldg(gx + at);
+    ay[y] = __ldg(gy + at);
+  }
+#pragma unroll
+  for (int y = 0; y < kCopySide; ++y) tile[warp * kCopySide + y][lane] = make_float2(ax[y], ay[y]);
+  __syncthreads();
+  const int count = min(kCopyPlanes, p.n_planes - q0);
+  for (int k = threadIdx.x; k < count * kCopySide * kCopySide; k += blockDim.x) {
+    const int y = k % kCopySide, x = k / kCopySide % kCopySide, i = k / (kCopySide * kCopySide);
+    if (x0 + x < v.ex && y0 + y < v.ey)
+      v.data[(static_cast<int64_t>(q0 + i) * v.ex + x0 + x) * v.ey + y0 + y] = tile[x * kCopySide + y][i];
+  }
+}
+
+// The projection from planes where a ray-mesh cell spans less than a mesh cell (P < kNarrow: the finest ray mesh, which
+// the resolution of the planes asks for): at most two mesh nodes per axis have a weight then.  The weights are separable,
+// so the block makes each row's and each column's two once per plane, and a thread has left what is its own: a load or two
+// and their sums, in place of the loops over candidates, which set the pace of the general kernel (about 180
+// instruction slots per warp and plane).  The sums are the same, term by term.
+constexpr double kNarrow = 0.99;
+constexpr int kBatch = 32;  // planes at a time
+
+__global__ void __launch_bounds__(kTileX * kTileY) raymesh_project_narrow_kernel(const __grid_constant__ ProjectParams p,
+                                                                                 float2* __restrict__ mesh, PlaneSlab v) {
+  __shared__ int2 s_base[kBatch];
+  __shared__ float2 s_frac[kBatch];
+  __shared__ float4 s_x[kBatch][kTileX];  // offset of the first row (integer bits), its weight and the next one's
+  __shared__ float2 s_wy[kBatch][kTileY];
+  __shared__ int s_y[kBatch][kTileY];
+  const int mx0 = v.row0 + blockIdx.y * kTileX, my0 = blockIdx.x * kTileY;
+  const int dmx = threadIdx.x / kTileY, dmy = threadIdx.x % kTileY;
+  float kx = 0.f, ky = 0.f;
+  for (int q0 = 0; q0 < p.n_planes; q0 += kBatch) {
+    const int count = min(kBatch, p.n_planes - q0);
+    __syncthreads();
+    if (threadIdx.x < count) {
+      const int q = q0 + threadIdx.x;
+      const double sx = p.qx[q] + mx0 * p.p[q], sy = p.qy[q] + my0 * p.p[q];
+      const double fx = floor(sx), fy = floor(sy);
+      s_base[threadIdx.x] = make_int2(static_cast<int>(fx) - v.x0, static_cast<int>(fy) - v.y0);
+      s_frac[threadIdx.x] = make_float2(static_cast<float>(sx - fx), static_cast<float>(sy - fy));
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < count * (kTileX + kTileY); e += blockDim.x) {
+      const int b = e / (kTileX + kTileY), t = e - b * (kTileX + kTileY);
+      const bool row = t < kTileX;
+      const float P = p.pf[q0 + b], inv = p.inv_p[q0 + b];
+      const float f = (row ? s_frac[b].x : s_frac[b].y) + (row ? t : t - kTileX) * P;
+      const int last = static_cast<int>(ceilf(f + P));
+      int first = 0;
+      float w0 = 0.f, w1 = 0.f;
+      for (int i = static_cast<int>(floorf(f - P)); i <= last; ++i) {
+        const float w = 1.f - fabsf(static_cast<float>(i) - f) * inv;
+        if (w <= 0.f) continue;
+        if (w0 > 0.f) {
+          w1 = w;
+        } else {
+          w0 = w;
+          first = i;
+        }
+      }
+      if (row) {
+        const int at = ((q0 + b) * v.ex + s_base[b].x + first) * v.ey;
+        s_x[b][t] = make_float4(__int_as_float(at), w0, w1, 0.f);
+      } else {
+        s_y[b][t - kTileX] = s_base[b].y + first;
+        s_wy[b][t - kTileX] = make_float2(w0, w1);
+      }
+    }
+    __syncthreads();
+#pragma unroll 4
+    for (int b = 0; b < count; ++b) {
+      const float4 x = s_x[b][dmx];
+      const float2 wy = s_wy[b][dmy];
+      const float2* __restrict__ at = v.data + (__float_as_int(x.x) + s_y[b][dmy]);
+      float sx = 0.f, sy = 0.f;
+      auto add = [&](float wx, float w, const float2* __restrict__ from) {
+        if (wx <= 0.f || w <= 0.f) return;
+        const float2 g = __ldg(from);
+        const float ww = wx * w;
+        sx += ww * g.x;
+        sy += ww * g.y;
+      };
+      add(x.y, wy.x, at);
+      add(x.y, wy.y, at + 1);
+      add(x.z, wy.x, at + v.ey);
+      add(x.z, wy.y, at + v.ey + 1);
+      kx += p.w[q0 + b] * sx;
+      ky += p.w[q0 + b] * sy;
+    }
+  }
+  const int mx = mx0 + dmx, my = my0 + dmy;
+  if (mx < p.n2d && my < p.n2d) mesh[static_cast<int64_t>(mx) * p.n2d + my] = make_float2(kx, ky);
+}
+
 template <bool TILED>
 __global__ void __launch_bounds__(kTileX * kTileY, 1) raymesh_project_kernel(const float* __restrict__ gx,
                                                                          const float* __restrict__ gy,
@@ -174,7 +301,9 @@ struct MeshView {
   const float2* k;  // nullptr: the half shell holds no plane (no kick)
   int n2d;
   double inv_x2d;
+  double fixed, fixed_half;  // 1 / x2d and n2d / 2 in units of 2^-47 cells (n2d is at most 2^15)
 };
+constexpr int kMeshBits = 47;
 
 struct RayMeshParams {
   MeshView m[2];
@@ -198,12 +327,15 @@ __device__ __forceinline__ float2 corner(const MeshView& m, int i, int j) {
 __device__ __forceinline__ MeshKick mesh_kick(const MeshView& m, double thx, double thy) {
   MeshKick h{0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
   if (m.k == nullptr) return h;
-  const double half = 0.5 * m.n2d;
-  const double ux = thx * m.inv_x2d + half, uy = thy * m.inv_x2d + half;
-  if (!(ux > -1.0 && ux < m.n2d && uy > -1.0 && uy < m.n2d)) return h;
-  const double flx = floor(ux), fly = floor(uy);
-  const int ix = static_cast<int>(flx), iy = static_cast<int>(fly);
-  const float fx = static_cast<float>(ux - flx), fy = static_cast<float>(uy - fly);
+  // Cell and fraction from one fixed-point number per axis with 47 bits after the point: an FP64 FMA and a conversion, where
+  // the plain form's floor, compares and differences take two FP64 lanes per SM several times as long.  The scaling is
+  // exact and a float's fraction has 24 bits, so that cell and fraction are those of mesh_locate; angles that are not
+  // finite or beyond the conversion's range end outside.
+  const long long kx = __double2ll_rd(fma(thx, m.fixed, m.fixed_half)), ky = __double2ll_rd(fma(thy, m.fixed, m.fixed_half));
+  const long long one = 1ll << kMeshBits, high = static_cast<long long>(m.n2d) << kMeshBits;
+  if (!(kx > -one && kx < high && ky > -one && ky < high)) return h;
+  const int ix = static_cast<int>(kx >> kMeshBits), iy = static_cast<int>(ky >> kMeshBits);
+  const float fx = __ll2float_rn(kx & (one - 1)) * 0x1p-47f, fy = __ll2float_rn(ky & (one - 1)) * 0x1p-47f;
   const float2 v00 = corner(m, ix, iy), v01 = corner(m, ix, iy + 1), v10 = corner(m, ix + 1, iy),
                v11 = corner(m, ix + 1, iy + 1);
   const float gx = 1.f - fx, gy = 1.f - fy;
@@ -654,6 +786,61 @@ static hrt_status filter_mesh(hrt_raymesh* rm, float2* mesh, int64_t n2d, cudaSt
   return cufft_check(cufftExecC2C(plan, c, c, CUFFT_INVERSE), "inverse");
 }
 
+// The rows of ray-mesh nodes from row0 on whose cells of all planes fit into `bytes` (a multiple of kTileX; all the rest if
+// they fit), as a slab; 0 if not even kTileX do.  Nodes within P of row m lie between q + (m - 1) P and q + (m + 1) P; two
+// cells to spare on either side.
+int64_t raymesh_slab(const ProjectParams& p, int64_t row0, int64_t bytes, PlaneSlab& v) {
+  auto extent = [&](const double* q, int64_t lo, int64_t hi, double& first) {
+    double a = INFINITY, b = -INFINITY;
+    for (int i = 0; i < p.n_planes; ++i) {
+      a = std::min(a, q[i] + (lo - 1) * p.p[i]);
+      b = std::max(b, q[i] + hi * p.p[i]);
+    }
+    first = std::floor(a) - 2.0;
+    return std::floor(b) + 4.0 - first;
+  };
+  double fx = 0.0, fy = 0.0;
+  const double ey = extent(p.qy, 0, p.n2d, fy), per_x = ey * p.n_planes * sizeof(float2);
+  int64_t rows = (p.n2d - row0 + kTileX - 1) / kTileX * kTileX;
+  double ex = extent(p.qx, row0, row0 + rows, fx);
+  while (ex * per_x > static_cast<double>(bytes)) {
+    if (rows <= kTileX) return 0;
+    rows = (rows / 2 + kTileX - 1) / kTileX * kTileX;
+    ex = extent(p.qx, row0, row0 + rows, fx);
+  }
+  v.x0 = static_cast<int>(fx);
+  v.y0 = static_cast<int>(fy);
+  v.ex = static_cast<int>(ex);
+  v.ey = static_cast<int>(ey);
+  v.row0 = static_cast<int>(row0);
+  return rows;
+}
+
+// The projection through copied planes where that pays and the workspace is to be had (done: it was made).
+static hrt_status project_planes(const float* gx, const float* gy, const ProjectParams& p, float2* mesh, cudaStream_t s,
+                                 bool& done) {
+  done = false;
+  PlaneSlab v{};
+  if (*std::max_element(p.p, p.p + p.n_planes) >= kNarrow) return HRT_OK;
+  if (static_cast<int64_t>(p.n2d) * p.n2d * p.n_planes < kSlabWork || raymesh_slab(p, 0, kSlabBytes, v) == 0) return HRT_OK;
+  const int64_t capacity = (static_cast<int64_t>(v.ex) + 2) * v.ey * p.n_planes * static_cast<int64_t>(sizeof(float2));
+  v.data = static_cast<float2*>(plane_workspace(static_cast<size_t>(capacity), s));
+  if (!v.data) return HRT_OK;
+  const int chunks = (p.n_planes + kCopyPlanes - 1) / kCopyPlanes;
+  for (int64_t row = 0, rows = 0; row < p.n2d; row += rows) {
+    rows = raymesh_slab(p, row, capacity, v);
+    if (rows == 0) break;
+    const unsigned tiles = static_cast<unsigned>(((v.ex + kCopySide - 1) / kCopySide) * ((v.ey + kCopySide - 1) / kCopySide));
+    raymesh_planes_kernel<<<tiles * chunks, 256, 0, s>>>(gx, gy, p, v);
+    const dim3 grid(static_cast<unsigned>((p.n2d + kTileY - 1) / kTileY), static_cast<unsigned>(rows / kTileX));
+    raymesh_project_narrow_kernel<<<grid, kTileX * kTileY, 0, s>>>(p, mesh, v);
+    done = row + rows >= p.n2d;
+  }
+  const cudaError_t launched = cudaGetLastError();
+  cudaFreeAsync(v.data, s);
+  return cuda_status(launched, "raymesh_project_kernel");
+}
+
 // Builds the filtered ray mesh of the half shell [chi_a, chi_b) in rm->mesh[h]; view.k == nullptr when the
 // shell holds no plane.
 static hrt_status build_mesh(hrt_raymesh* rm, int h, const float* gx, const float* gy, const float* gz,
@@ -666,6 +853,8 @@ static hrt_status build_mesh(hrt_raymesh* rm, int h, const float* gx, const floa
   HRT_TRY(plane_table(g, chi_a, chi_b, a_ref, omega_m, x2d, n2d, p));
   view.n2d = static_cast<int>(n2d);
   view.inv_x2d = 1.0 / x2d;
+  view.fixed = std::ldexp(view.inv_x2d, kMeshBits);
+  view.fixed_half = std::ldexp(0.5 * static_cast<double>(n2d), kMeshBits);
   view.k = nullptr;
   if (p.n_planes == 0) return HRT_OK;
   HRT_TRY(ensure_mesh(rm, h, n2d * n2d, s));
@@ -674,10 +863,15 @@ static hrt_status build_mesh(hrt_raymesh* rm, int h, const float* gx, const floa
   if (p.tiled) {
     if (!gz) return fail(HRT_ERR_INVALID_ARG, "light-cone tiling needs the third gradient component");
     raymesh_project_kernel<true><<<grid, kTileX * kTileY, 0, s>>>(gx, gy, gz, p, mesh);
+    HRT_LAUNCHED("raymesh_project_kernel");
   } else {
-    raymesh_project_kernel<false><<<grid, kTileX * kTileY, 0, s>>>(gx, gy, gz, p, mesh);
+    bool done = false;
+    HRT_TRY(project_planes(gx, gy, p, mesh, s, done));
+    if (!done) {
+      raymesh_project_kernel<false><<<grid, kTileX * kTileY, 0, s>>>(gx, gy, gz, p, mesh);
+      HRT_LAUNCHED("raymesh_project_kernel");
+    }
   }
-  HRT_LAUNCHED("raymesh_project_kernel");
   HRT_TRY(filter_mesh(rm, mesh, n2d, s));
   view.k = mesh;
   return HRT_OK;
