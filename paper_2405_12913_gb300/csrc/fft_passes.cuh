@@ -210,7 +210,7 @@ struct Dfts<R, 0> {
 };
 
 // ---- lines of a warp ----------------------------------------------------------------------------------------
-// P line pairs per warp and W warps per tile block: 4 pairs (8 kz) per tile row.
+// P line pairs per warp and W warps per tile: 4 pairs (8 kz) per tile row.
 template <int R1>
 struct Cfg {
   static constexpr int N = 32 * R1;
@@ -498,12 +498,28 @@ struct Tile {
   }
 };
 
-// The block's tile buffer (1024-byte aligned) and one tile's copy into it; load(dst, bar) issues the copies.  False
-// after a timed-out wait, with the copies given another bounded wait to land before the block ends.
-template <int R1, class Load>
-__device__ __forceinline__ bool fetch_tile(uint32_t buf, uint64_t* bar, int* __restrict__ err, Load load) {
-  const uint32_t b = smem_u32(bar);
-  if (threadIdx.x == 0) {
+// A warp's tile within its block of G tiles: the tile's number, buffer (1024-byte aligned) and barrier, the warp among the
+// tile's and the thread that issues its copies.
+template <int R1, int G = 1>
+struct Place {
+  using C = Cfg<R1>;
+  const unsigned char* raw;
+  uint64_t* bars;
+  __device__ __forceinline__ static int group() { return G == 1 ? 0 : static_cast<int>(threadIdx.x) / C::Threads; }
+  __device__ __forceinline__ unsigned tile() const { return blockIdx.x * G + group(); }
+  __device__ __forceinline__ uint32_t base() const { return (smem_u32(raw) + 1023u) & ~1023u; }
+  __device__ __forceinline__ uint32_t buf() const { return base() + group() * C::TileBytes; }
+  __device__ __forceinline__ uint32_t bar() const { return smem_u32(bars + group()); }
+  __device__ __forceinline__ int warp() const { return static_cast<int>(threadIdx.x >> 5) - group() * C::W; }
+  __device__ __forceinline__ bool leader() const { return (G == 1 ? threadIdx.x : threadIdx.x % C::Threads) == 0; }
+};
+
+// One tile's copy into its buffer; load(dst, bar) issues the copies.  False for the whole block after a timed-out wait, with
+// the copies given another bounded wait to land before the block ends.
+template <int R1, int G, class Load>
+__device__ __forceinline__ bool fetch_tile(const Place<R1, G>& at, int* __restrict__ err, Load load) {
+  const uint32_t b = at.bar(), buf = at.buf();
+  if (at.leader()) {
     mbar_init(b, 1);
     fence_mbar_init();
     mbar_expect_tx(b, Cfg<R1>::TileBytes);
@@ -512,35 +528,30 @@ __device__ __forceinline__ bool fetch_tile(uint32_t buf, uint64_t* bar, int* __r
   __syncthreads();
   const bool got = mbar_wait(b, 0u);
   if (__syncthreads_and(got)) return true;
-  if (threadIdx.x == 0) {
+  if (at.leader()) {
     atomicOr(err, kFftTimeout);
     mbar_wait(b, 0u);
   }
   return false;
 }
 
-// The next tile into the block's buffer once every warp is done with the last one; phase: its number, from 1.
-template <int R1, class Load>
-__device__ __forceinline__ bool fetch_next(uint32_t buf, uint64_t* bar, uint32_t phase, int* __restrict__ err, Load load) {
-  const uint32_t b = smem_u32(bar);
+// The next tile into the buffer once every warp is done with the last one; phase: its number, from 1.
+template <int R1, int G, class Load>
+__device__ __forceinline__ bool fetch_next(const Place<R1, G>& at, uint32_t phase, int* __restrict__ err, Load load) {
+  const uint32_t b = at.bar(), buf = at.buf();
   fence_async_shared();
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (at.leader()) {
     mbar_expect_tx(b, Cfg<R1>::TileBytes);
     load(buf, b);
   }
   const bool got = mbar_wait(b, phase & 1u);
   if (__syncthreads_and(got)) return true;
-  if (threadIdx.x == 0) {
+  if (at.leader()) {
     atomicOr(err, kFftTimeout);
     mbar_wait(b, phase & 1u);
   }
   return false;
-}
-
-__device__ __forceinline__ uint32_t tile_buffer(const unsigned char* raw) {
-  const uint32_t a = smem_u32(raw);
-  return (a + 1023u) & ~1023u;
 }
 
 // Signed frequency times kf, 0 at the Nyquist frequency.
@@ -561,11 +572,12 @@ __global__ void __launch_bounds__(Cfg<R1>::Threads, Cfg<R1>::Blocks)
   using C = Cfg<R1>;
   using T = Tile<R1>;
   extern __shared__ unsigned char raw[];
-  __shared__ uint64_t bar;
-  const uint32_t buf = tile_buffer(raw);
-  const int x = blockIdx.x / blocks_kz, kb = blockIdx.x - x * blocks_kz;
-  if (!fetch_tile<R1>(buf, &bar, err, [&](uint32_t d, uint32_t b) { T::load_plane(d, &f.in[blockIdx.y], x, kb, b); })) return;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  __shared__ uint64_t bars[1];
+  const Place<R1> here{raw, bars};
+  const uint32_t buf = here.buf();
+  const int x = here.tile() / blocks_kz, kb = here.tile() - x * blocks_kz;
+  if (!fetch_tile(here, err, [&](uint32_t d, uint32_t b) { T::load_plane(d, &f.in[blockIdx.y], x, kb, b); })) return;
+  const int lane = threadIdx.x & 31, warp = here.warp();
   const TileAddr at{buf, warp * C::P};
   C2 v[32];
 #pragma unroll
@@ -578,7 +590,7 @@ __global__ void __launch_bounds__(Cfg<R1>::Threads, Cfg<R1>::Blocks)
   for (int k2 = 0; k2 < 32; ++k2) sts(at(pb, k1 + R1 * k2), v[slot<32>(k2)]);
   fence_async_shared();
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (here.leader()) {
     T::store_column(&f.out[blockIdx.y], buf, x, kb);
     bulk_commit();
     bulk_wait_read_all();
@@ -599,13 +611,14 @@ __global__ void __launch_bounds__(Cfg<R1>::Threads, Cfg<R1>::Blocks)
   using C = Cfg<R1>;
   using T = Tile<R1>;
   extern __shared__ unsigned char raw[];
-  __shared__ uint64_t bar;
-  const uint32_t buf = tile_buffer(raw);
-  const unsigned tile = blockIdx.x / static_cast<unsigned>(jobs.jobs);
-  const int job = blockIdx.x - tile * jobs.jobs;
+  __shared__ uint64_t bars[1];
+  const Place<R1> here{raw, bars};
+  const uint32_t buf = here.buf();
+  const unsigned tile = here.tile() / static_cast<unsigned>(jobs.jobs);
+  const int job = here.tile() - tile * jobs.jobs;
   const int x = tile / blocks_kz, kb = tile - x * blocks_kz;
-  if (!fetch_tile<R1>(buf, &bar, err, [&](uint32_t d, uint32_t b) { T::load_column(d, &jobs.in[job], x, kb, b); })) return;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (!fetch_tile(here, err, [&](uint32_t d, uint32_t b) { T::load_column(d, &jobs.in[job], x, kb, b); })) return;
+  const int lane = threadIdx.x & 31, warp = here.warp();
   const TileAddr at{buf, warp * C::P};
   const int kind = job % 3;
   C2 v[32];
@@ -633,7 +646,7 @@ __global__ void __launch_bounds__(Cfg<R1>::Threads, Cfg<R1>::Blocks)
   for (int k2 = 0; k2 < 32; ++k2) sts(at(pb, k1 + R1 * k2), swapped(v[slot<32>(k2)]));
   fence_async_shared();
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (here.leader()) {
     T::store_plane(&jobs.out[job], buf, x, kb);
     bulk_commit();
     bulk_wait_read_all();
@@ -647,11 +660,12 @@ __global__ void __launch_bounds__(Cfg<R1>::Threads, Cfg<R1>::Blocks)
                         float2* __restrict__ out, int* __restrict__ err) {
   using C = Cfg<R1>;
   extern __shared__ unsigned char raw[];
-  __shared__ uint64_t bar;
-  const uint32_t buf = tile_buffer(raw);
-  const int ky = blockIdx.x / blocks_kz, kb = blockIdx.x - ky * blocks_kz;
-  if (!fetch_tile<R1>(buf, &bar, err, [&](uint32_t d, uint32_t b) { Tile<R1>::load_line(d, &in, ky, kb, b); })) return;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  __shared__ uint64_t bars[1];
+  const Place<R1> here{raw, bars};
+  const uint32_t buf = here.buf();
+  const int ky = here.tile() / blocks_kz, kb = here.tile() - ky * blocks_kz;
+  if (!fetch_tile(here, err, [&](uint32_t d, uint32_t b) { Tile<R1>::load_line(d, &in, ky, kb, b); })) return;
+  const int lane = threadIdx.x & 31, warp = here.warp();
   const TileAddr at{buf, warp * C::P};
   C2 v[32];
 #pragma unroll
@@ -693,31 +707,43 @@ struct XJobs {
 // warps per SM.  Other places for it were slower: made again by a second block (three blocks of 168 registers per SM)
 // 3.77 ms, kept in the V spectrum's own lines in L2 3.85 ms.
 constexpr int kKeep = 9;
-template <int R1>
+// With a learned factor (MANY) a block holds as many tiles as give it four warps: they stay together at the block's barriers and
+// share their instruction fetches, where blocks of one or two warps, at different places of a larger kernel, wait for theirs.
+// Five fields, before and now: 512^3 4.01 -> 3.19 ms, 384^3 1.70 -> 1.46 ms, 256^3 508 -> 453 us; the plain kernels gain nothing
+// by it (192^3 137 and 144 us).
+template <int R1, bool MANY>
 struct XCfg {
+  static constexpr int G = MANY ? 4 / Cfg<R1>::W : 1;
+  static constexpr int Threads = G * Cfg<R1>::Threads;
+  static constexpr int Blocks = 8 / (Cfg<R1>::W * G);
   static constexpr int Stash = 32 - kKeep;
-  static constexpr int Bytes = Cfg<R1>::TileBytes + Cfg<R1>::W * Stash * 512 + 1024;
+  static constexpr int Bytes = G * (Cfg<R1>::TileBytes + Cfg<R1>::W * Stash * 512) + 1024;
+  // this warp's stash, behind the block's tiles
+  __device__ __forceinline__ static uint32_t stash(uint32_t base) {
+    return base + G * Cfg<R1>::TileBytes + (threadIdx.x >> 5) * (Stash * 512);
+  }
 };
 
 template <int R1, bool LEARNED>
-__global__ void __launch_bounds__(Cfg<R1>::Threads, 8 / Cfg<R1>::W)
+__global__ void __launch_bounds__(XCfg<R1, LEARNED>::Threads, XCfg<R1, LEARNED>::Blocks)
     fft_x_kernel(const __grid_constant__ XJobs jobs, const float2* __restrict__ tw, int blocks_kz, float kf, float scale,
                  int* __restrict__ err) {
   using C = Cfg<R1>;
   using T = Tile<R1>;
-  constexpr int N = C::N, S = XCfg<R1>::Stash;
+  constexpr int N = C::N, S = XCfg<R1, LEARNED>::Stash, G = XCfg<R1, LEARNED>::G;
   extern __shared__ unsigned char raw[];
-  __shared__ uint64_t bar;
-  const uint32_t buf = tile_buffer(raw);
-  const unsigned tile = blockIdx.x / static_cast<unsigned>(jobs.sets);
-  const int set = blockIdx.x - tile * jobs.sets;
+  __shared__ uint64_t bars[G];
+  const Place<R1, G> here{raw, bars};
+  const uint32_t buf = here.buf();
+  const unsigned tile = here.tile() / static_cast<unsigned>(jobs.sets);
+  const int set = here.tile() - tile * jobs.sets;
   // 16 consecutive tiles share a region: ky mod 16 fastest
   const unsigned region = tile >> 4;
   const int kg = region / blocks_kz, kb = region - kg * blocks_kz, ky = kg * 16 + (tile & 15);
-  if (!fetch_tile<R1>(buf, &bar, err, [&](uint32_t d, uint32_t b) { T::load_line(d, &jobs.in, ky, kb, b); })) return;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (!fetch_tile(here, err, [&](uint32_t d, uint32_t b) { T::load_line(d, &jobs.in, ky, kb, b); })) return;
+  const int lane = threadIdx.x & 31, warp = here.warp();
   const TileAddr at{buf, warp * C::P};
-  const uint32_t stash = buf + C::TileBytes + warp * (S * 512) + lane * 16;
+  const uint32_t stash = XCfg<R1, LEARNED>::stash(here.base()) + lane * 16;
   const int lb = Cfg<R1>::second(lane), pb = lb / R1, k1 = lb % R1;
   C2 u[32], keep[kKeep];
   {
@@ -779,7 +805,7 @@ __global__ void __launch_bounds__(Cfg<R1>::Threads, 8 / Cfg<R1>::W)
       for (int m = 0; m < R1; ++m) sts(at(p, lane + 32 * m), swapped(u[p * R1 + slot<R1>(m)]));
     fence_async_shared();
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (here.leader()) {
       T::store_line(&jobs.out[2 * set + component], buf, ky, kb);
       bulk_commit();
     }
@@ -790,11 +816,11 @@ __global__ void __launch_bounds__(Cfg<R1>::Threads, 8 / Cfg<R1>::W)
 #pragma unroll
   for (int i = 0; i < kKeep; ++i) u[S + i] = keep[i];
   inverse_first<R1>(u, tw, lane);
-  if (threadIdx.x == 0) bulk_wait_read_all();  // the x component has left the tile
+  if (here.leader()) bulk_wait_read_all();  // the x component has left the tile
   __syncthreads();
   inverse_second<R1>(u, at, lane);
   put(1);
-  if (threadIdx.x == 0) bulk_wait_read_all();
+  if (here.leader()) bulk_wait_read_all();
 }
 
 // Transpose of the x-pass for one filter set: out = IFFT_x(-i c (d_x FFT_x(in[0]) + FFT_x(d_y in[1] + d_z in[2]))), the
@@ -806,26 +832,27 @@ struct XAdjoint {
 };
 
 template <int R1, bool LEARNED>
-__global__ void __launch_bounds__(Cfg<R1>::Threads, 8 / Cfg<R1>::W)
+__global__ void __launch_bounds__(Cfg<R1>::Threads, XCfg<R1, false>::Blocks)
     fft_x_adjoint_kernel(const __grid_constant__ XAdjoint f, const float2* __restrict__ tw, int blocks_kz, float kf, float scale,
                          int* __restrict__ err) {
   using C = Cfg<R1>;
   using T = Tile<R1>;
-  constexpr int N = C::N, S = XCfg<R1>::Stash;
+  constexpr int N = C::N, S = XCfg<R1, false>::Stash;
   extern __shared__ unsigned char raw[];
-  __shared__ uint64_t bar;
-  const uint32_t buf = tile_buffer(raw);
-  const unsigned region = blockIdx.x >> 4;
-  const int kg = region / blocks_kz, kb = region - kg * blocks_kz, ky = kg * 16 + (blockIdx.x & 15);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  __shared__ uint64_t bars[1];
+  const Place<R1> here{raw, bars};
+  const uint32_t buf = here.buf();
+  const unsigned region = here.tile() >> 4;
+  const int kg = region / blocks_kz, kb = region - kg * blocks_kz, ky = kg * 16 + (here.tile() & 15);
+  const int lane = threadIdx.x & 31, warp = here.warp();
   const TileAddr at{buf, warp * C::P};
-  const uint32_t stash = buf + C::TileBytes + warp * (S * 512) + lane * 16;
+  const uint32_t stash = XCfg<R1, false>::stash(here.base()) + lane * 16;
   const int lb = C::second(lane), pb = lb / R1, k1 = lb % R1;
   auto load = [&](const CUtensorMap* m) {
     return [=](uint32_t d, uint32_t b) { T::load_line(d, m, ky, kb, b); };
   };
   C2 v[32], keep[kKeep];
-  if (!fetch_tile<R1>(buf, &bar, err, load(&f.in[1]))) return;
+  if (!fetch_tile(here, err, load(&f.in[1]))) return;
   const u64 dy = both(derivative(ky, N, kf));
 #pragma unroll
   for (int p = 0; p < C::P; ++p)
@@ -834,7 +861,7 @@ __global__ void __launch_bounds__(Cfg<R1>::Threads, 8 / Cfg<R1>::W)
       const C2 x = lds(at(p, lane + 32 * m));
       v[p * R1 + m] = {mul2(x.re, dy), mul2(x.im, dy)};
     }
-  if (!fetch_next<R1>(buf, &bar, 1, err, load(&f.in[2]))) return;
+  if (!fetch_next(here, 1, err, load(&f.in[2]))) return;
 #pragma unroll
   for (int p = 0; p < C::P; ++p) {
     const int kz = kb * 8 + 2 * (warp * C::P + p);
@@ -851,7 +878,7 @@ __global__ void __launch_bounds__(Cfg<R1>::Threads, 8 / Cfg<R1>::W)
   for (int i = 0; i < S; ++i) sts(stash + i * 512, v[slot<32>(i)]);
 #pragma unroll
   for (int i = 0; i < kKeep; ++i) keep[i] = v[slot<32>(S + i)];
-  if (!fetch_next<R1>(buf, &bar, 2, err, load(&f.in[0]))) return;
+  if (!fetch_next(here, 2, err, load(&f.in[0]))) return;
 #pragma unroll
   for (int p = 0; p < C::P; ++p)
 #pragma unroll
@@ -887,7 +914,7 @@ __global__ void __launch_bounds__(Cfg<R1>::Threads, 8 / Cfg<R1>::W)
     for (int m = 0; m < R1; ++m) sts(at(p, lane + 32 * m), swapped(u[p * R1 + slot<R1>(m)]));
   fence_async_shared();
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (here.leader()) {
     T::store_line(&f.out, buf, ky, kb);
     bulk_commit();
     bulk_wait_read_all();
@@ -927,10 +954,15 @@ hrt_status Passes<R1>::x_pass(const FftPlan& p, double box, double pref, const F
   for (int i = 0; i < 2 * j.sets; ++i) j.out[i] = p.x_out[i];
   j.set[0] = a;
   j.set[1] = b ? *b : a;
-  const auto kernel = a.g || (b && b->g) ? fft_x_kernel<R1, true> : fft_x_kernel<R1, false>;
-  HRT_TRY(reserve(kernel, XCfg<R1>::Bytes));
+  const bool learned = a.g || (b && b->g);
+  const auto kernel = learned ? fft_x_kernel<R1, true> : fft_x_kernel<R1, false>;
+  using Many = XCfg<R1, true>;
+  using One = XCfg<R1, false>;
+  const int bytes = learned ? Many::Bytes : One::Bytes, threads = learned ? Many::Threads : One::Threads;
+  const int blocks = C::N * kb * j.sets / (learned ? Many::G : One::G);
+  HRT_TRY(reserve(kernel, bytes));
   const double scale = -pref / (static_cast<double>(C::N) * C::N * C::N);
-  kernel<<<C::N * kb * j.sets, C::Threads, XCfg<R1>::Bytes, s>>>(
+  kernel<<<blocks, threads, bytes, s>>>(
       j, p.tw, kb, static_cast<float>(2.0 * M_PI / box), static_cast<float>(scale), p.err);
   HRT_LAUNCHED("fft_x_kernel");
   return HRT_OK;
@@ -995,9 +1027,9 @@ hrt_status Passes<R1>::adjoint(const FftPlan& p, double box, double pref, const 
   HRT_LAUNCHED("fft_y_kernel");
   XAdjoint x{{q.x_in[0], q.x_in[1], q.x_in[2]}, q.x_out, a};
   const auto kernel = a.g ? fft_x_adjoint_kernel<R1, true> : fft_x_adjoint_kernel<R1, false>;
-  HRT_TRY(reserve(kernel, XCfg<R1>::Bytes));
+  HRT_TRY(reserve(kernel, XCfg<R1, false>::Bytes));
   const float kf = static_cast<float>(2.0 * M_PI / box);
-  kernel<<<C::N * kb, C::Threads, XCfg<R1>::Bytes, s>>>(
+  kernel<<<C::N * kb, C::Threads, XCfg<R1, false>::Bytes, s>>>(
       x, p.tw, kb, kf, static_cast<float>(-pref / (static_cast<double>(C::N) * C::N * C::N)), p.err);
   HRT_LAUNCHED("fft_x_adjoint_kernel");
   YJobs y{};
