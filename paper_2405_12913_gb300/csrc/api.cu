@@ -1716,7 +1716,8 @@ hrt_status hrt_workspace_bytes(const hrt_config* cfg, int64_t n_rays, size_t* by
   if (!bytes || n_rays < 0) return fail(HRT_ERR_INVALID_ARG, "bad arguments");
   const size_t n = cfg->n_mesh, mesh = n * n * n * sizeof(float), np = cfg->n_side * cfg->n_side * cfg->n_side;
   size_t b = 6 * np * sizeof(float) + mesh * (4 + cfg->ray_fields);
-  size_t work = 2 * spectrum_bytes(cfg->n_mesh);  // cuFFT, and the further spectra of the FFT passes in its place
+  // cuFFT, and the further spectra of the FFT passes in its place
+  size_t work = (cfg->n_mesh <= kBatchSide ? 3 : 2) * spectrum_bytes(cfg->n_mesh);
   if (fft_supported(cfg->n_mesh))
     work = std::max(work, fft_spectrum_bytes(cfg->n_mesh) * split_spectra(cfg->n_mesh, cfg->ray_fields));
   b += spectrum_alloc(cfg->n_mesh) * (1 + 3 + cfg->ray_fields) + work;
