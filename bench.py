@@ -259,12 +259,13 @@ def run_gpu(args, W, world, rank, local):
     disp0, mom0, _, _ = ctx.hrt_read_particles()
     grid = W.reverse_grid
     slots = {s: i for i, s in enumerate(W.source_steps)}
-    # own kernels per ray step: the direct gather is one launch; the ray mesh is, per half shell, the projection
-    # and the filter (around cuFFT's transforms), then the ray kernel
-    ray_launches = 1
+    # own kernels per ray step: the direct gather is three launches (the rays' bounds, the node planes, the step; the last
+    # alone for a small bundle); the ray mesh is, per half shell, the copy of its planes, the projection and the filter
+    # (around cuFFT's transforms), then the ray kernel
+    ray_launches = 3 if W.n_rays >= 1 << 18 else 1
     if args.kick == "mesh":
         ctx.hrt_set_ray_mesh(raymesh_config(hrt, W))
-        ray_launches = 5
+        ray_launches = 7 if W.n_rays >= 1 << 18 else 5
 
     # own kernels per Poisson solve: the FFT passes along z, y, x and back, or the k-space kernel between cuFFT plans
     solve_launches = 5 if own_fft(W) else 1
