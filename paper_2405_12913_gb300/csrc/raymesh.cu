@@ -91,8 +91,10 @@ struct PlaneSlab {
 };
 // Bytes of a slab: the planes stay in L2 between the copy and the projection; a larger mesh goes in slabs of rows.
 constexpr int64_t kSlabBytes = int64_t{60} << 20;
-// Ray-mesh nodes times planes from which a second launch per half shell pays.
-constexpr int64_t kSlabWork = 1 << 20;
+// Ray-mesh nodes times planes above which the copy and the workspace's allocation pay.  The kick of a half shell with the planes
+// and from the fields: 512^2 nodes and 16 planes 61 and 50 us, 32 planes 75 and 77 (the line), 64 planes 108 and 133; 1024^2 nodes
+// and 8 planes (the line) 95 and 90, 16 planes 113 and 133, 32 planes 173 and 227 us.
+constexpr int64_t kSlabWork = 1 << 23;
 
 // A block copies 32 planes of 8 x 8 cells: a lane per plane, so that a warp reads a column's run of z as it lies, and rows of
 // y leave through shared memory.
@@ -822,7 +824,7 @@ static hrt_status project_planes(const float* gx, const float* gy, const Project
   done = false;
   PlaneSlab v{};
   if (*std::max_element(p.p, p.p + p.n_planes) >= kNarrow) return HRT_OK;
-  if (static_cast<int64_t>(p.n2d) * p.n2d * p.n_planes < kSlabWork || raymesh_slab(p, 0, kSlabBytes, v) == 0) return HRT_OK;
+  if (static_cast<int64_t>(p.n2d) * p.n2d * p.n_planes <= kSlabWork || raymesh_slab(p, 0, kSlabBytes, v) == 0) return HRT_OK;
   const int64_t capacity = (static_cast<int64_t>(v.ex) + 2) * v.ey * p.n_planes * static_cast<int64_t>(sizeof(float2));
   v.data = static_cast<float2*>(plane_workspace(static_cast<size_t>(capacity), s));
   if (!v.data) return HRT_OK;
