@@ -261,7 +261,12 @@ __device__ __forceinline__ HalfKick half_kick_planes(const RayStepParams& p, int
   const long long kx = __double2ll_rd(fma(fixed_r, th_x, p.fixed_obs_x)), ky = __double2ll_rd(fma(fixed_r, th_y, p.fixed_obs_y));
   const int cx = static_cast<int>(kx >> 32), cy = static_cast<int>(ky >> 32);
   const float fbx = static_cast<float>(static_cast<unsigned>(kx)) * 0x1p-32f, fby = static_cast<float>(static_cast<unsigned>(ky)) * 0x1p-32f;
-  const int bx = cx - b.x0, by = cy - b.y0;
+  // Cells within 2^29 of the origin, looked at before anything is compared with them: the box starts within 1e9, so that no
+  // sum of cells leaves int.  Angles that are not finite, or out of the conversion's range, saturate and end outside.
+  constexpr unsigned kCells = 1u << 29;
+  const bool near = static_cast<unsigned>(cx) + kCells < 2 * kCells && static_cast<unsigned>(cy) + kCells < 2 * kCells;
+  const int bx = static_cast<int>(static_cast<unsigned>(cx) - static_cast<unsigned>(b.x0)),
+            by = static_cast<int>(static_cast<unsigned>(cy) - static_cast<unsigned>(b.y0));
   const float tx = static_cast<float>(th_x), ty = static_cast<float>(th_y);
   auto inside = [&](float dr) {
     const float px = fbx + dr * tx, py = fby + dr * ty;
@@ -269,15 +274,15 @@ __device__ __forceinline__ HalfKick half_kick_planes(const RayStepParams& p, int
     const int x = bx + static_cast<int>(floorf(px)), y = by + static_cast<int>(floorf(py));
     return x >= 0 && x + 1 < b.rx && y >= 0 && y + 1 < b.ry;
   };
-  // (angles that are not finite, or out of the conversion's range, end outside)
-  if (abs(cx + 1) > (1 << 30) || abs(cy + 1) > (1 << 30) || !inside(node[j0].x) || !inside(node[j1 - 1].x))
+  if (!near || !inside(node[j0].x) || !inside(node[j1 - 1].x))
     return half_kick(p, j0, j1, th_x, th_y, ref_r, gx, gy);
   // floor as an integer from the bits of floor + 1.5 2^23 (the conversion unit is slow); the offset of those bits is taken
   // off here once
   constexpr float kMagic = 12582912.f;
   constexpr unsigned kMagicBits = 0x4b400000u;
   const int plane = b.rx * b.ry;
-  const unsigned offset = static_cast<unsigned>(by * b.rx + bx) - kMagicBits * static_cast<unsigned>(b.rx + 1);
+  const unsigned offset = static_cast<unsigned>(by) * static_cast<unsigned>(b.rx) + static_cast<unsigned>(bx) -
+                          kMagicBits * static_cast<unsigned>(b.rx + 1);
   const float2* __restrict__ at = planes + static_cast<int64_t>(j0) * plane;
   // both components of a corner, (d_x phi, d_y phi), side by side
   u64 k = 0, jx = 0, jy = 0;
