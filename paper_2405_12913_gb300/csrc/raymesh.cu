@@ -332,10 +332,15 @@ __device__ __forceinline__ MeshKick mesh_kick(const MeshView& m, double thx, dou
   // Cell and fraction from one fixed-point number per axis with 47 bits after the point: an FP64 FMA and a conversion, where
   // the plain form's floor, compares and differences take two FP64 lanes per SM several times as long.  The scaling is
   // exact and a float's fraction has 24 bits, so that cell and fraction are those of mesh_locate; angles that are not
-  // finite or beyond the conversion's range end outside.
-  const long long kx = __double2ll_rd(fma(thx, m.fixed, m.fixed_half)), ky = __double2ll_rd(fma(thy, m.fixed, m.fixed_half));
+  // finite or beyond the conversion's range end outside.  A position above -1 by less than 2^-47 rounds down to -1 but
+  // is inside: there the number before the conversion decides (its bits, without an FP64 lane).
+  const double sx = fma(thx, m.fixed, m.fixed_half), sy = fma(thy, m.fixed, m.fixed_half);
+  const long long kx = __double2ll_rd(sx), ky = __double2ll_rd(sy);
   const long long one = 1ll << kMeshBits, high = static_cast<long long>(m.n2d) << kMeshBits;
-  if (!(kx > -one && kx < high && ky > -one && ky < high)) return h;
+  auto inside = [&](double s, long long k) {
+    return k < high && (k > -one || (k == -one && __double_as_longlong(s) != __double_as_longlong(-0x1p47)));
+  };
+  if (!inside(sx, kx) || !inside(sy, ky)) return h;
   const int ix = static_cast<int>(kx >> kMeshBits), iy = static_cast<int>(ky >> kMeshBits);
   const float fx = __ll2float_rn(kx & (one - 1)) * 0x1p-47f, fy = __ll2float_rn(ky & (one - 1)) * 0x1p-47f;
   const float2 v00 = corner(m, ix, iy), v01 = corner(m, ix, iy + 1), v10 = corner(m, ix + 1, iy),
