@@ -663,8 +663,9 @@ hrt_status launch_rays_init(const hrt_rays& rays, const double* theta0, cudaStre
 // atomics per mode, most lanes of a warp on the same bin, took 880 us at m = 2048.  A warp now takes 256 columns of
 // the rows nx and -nx, whose geometry is the same; a lane's modes climb through the bins, so it adds in registers, and
 // what lanes hold goes to shared memory, summed over the warp, where a bin ends and at the end: 70 us with a shared-memory
-// atomic per lane there, 34 us with the sum.  |n| is a float
-// square root with its residual (2^-46), squares are float pairs and partial sums become FP64 when they leave the lane.
+// atomic per lane there, 34 us with the sum.  A lane's sums of |n| and of the squares are three floats each, which round less
+// than FP64; they become FP64 when they leave the lane.  (With two floats each P was off by up to 4.6e-15 from the sums
+// of the same spectrum in 80 bits, with FP64 by 1.2e-15, now by 0.7e-15; a call takes the same time with two and three.)
 // ---------------------------------------------------------------------------------------------------------
 constexpr int kBinColumns = 256;
 
@@ -672,12 +673,46 @@ constexpr int kBinColumns = 256;
 __device__ __forceinline__ bool moderate(float x) { return x == 0.f || (fabsf(x) > 1e-12f && fabsf(x) < 1e15f); }
 __device__ __forceinline__ bool moderate(float2 z) { return moderate(z.x) && moderate(z.y); }
 
-// hi + lo += scale x^2 with the rounding errors kept; scale a power of two.
-__device__ __forceinline__ void add_square(float x, float scale, float& hi, float& lo) {
-  const float sx = scale * x, q = __fmul_rn(sx, x), e = __fmaf_rn(sx, x, -q);
-  const float sum = __fadd_rn(hi, q), back = __fsub_rn(sum, hi);
-  lo += __fadd_rn(__fsub_rn(hi, __fsub_rn(sum, back)), __fsub_rn(q, back)) + e;
-  hi = sum;
+// A sum in three floats of falling size: what a float sum rounds away goes to the next, so that 2^-70 of it is lost at
+// most, less than in FP64.
+struct Sum3 {
+  float hi, mid, lo;
+};
+__device__ __forceinline__ float two_sum(float a, float b, float& rounded) {
+  const float s = __fadd_rn(a, b), back = __fsub_rn(s, a);
+  rounded = __fadd_rn(__fsub_rn(a, __fsub_rn(s, back)), __fsub_rn(b, back));
+  return s;
+}
+// x to the middle of the sum: a rounding error of what went on top
+__device__ __forceinline__ void add_small(Sum3& s, float x) {
+  float e;
+  s.mid = two_sum(s.mid, x, e);
+  s.lo += e;
+}
+__device__ __forceinline__ void add_to(Sum3& s, float x) {
+  float e;
+  s.hi = two_sum(s.hi, x, e);
+  add_small(s, e);
+}
+__device__ __forceinline__ double value(const Sum3& s) { return static_cast<double>(s.hi) + (static_cast<double>(s.mid) + s.lo); }
+
+// s += scale x^2; scale a power of two.
+__device__ __forceinline__ void add_square(Sum3& s, float x, float scale) {
+  const float sx = scale * x, q = __fmul_rn(sx, x);
+  add_to(s, q);
+  add_small(s, __fmaf_rn(sx, x, -q));
+}
+
+// s += modes sqrt(n2); modes a power of two, n2 > 0.  The float root, then the residual's share of it to first order as
+// a quotient with its own residual, and the second order: 2^-70.
+__device__ __forceinline__ void add_root(Sum3& s, int n2, int modes) {
+  const float a = static_cast<float>(n2), root = sqrtf(a), twice = 2.f * root;
+  float left;
+  const float r = two_sum(__fmaf_rn(-root, root, a), static_cast<float>(n2 - static_cast<int>(a)), left);
+  const float c = r / twice, rest = (__fmaf_rn(-twice, c, r) + left - c * c) / twice;
+  add_to(s, root * modes);
+  add_small(s, c * modes);
+  s.lo += rest * modes;
 }
 
 __global__ void __launch_bounds__(256) power_bin_kernel(const float2* __restrict__ spec, int m, double ell_scale,
@@ -718,18 +753,17 @@ __global__ void __launch_bounds__(256) power_bin_kernel(const float2* __restrict
         }
       }
     }
-    // squares as float pairs (2^-48) where no square or its rounding error can leave float's range, else in FP64
+    // squares in floats where no square or its rounding error can leave float's range, else in FP64
     bool small = true;
 #pragma unroll
     for (int i = 0; i < kBinColumns / 32; ++i) small = small && moderate(u[i]) && moderate(v[i]);
     const bool plain = __all_sync(0xffffffffu, small);
     double power = 0.0;
-    float pw_hi = 0.f, pw_lo = 0.f, ell_hi = 0.f, ell_lo = 0.f;
+    Sum3 squares{0.f, 0.f, 0.f}, roots{0.f, 0.f, 0.f};
     int count = 0;
     // what the lanes with `out` hold of their bins, summed over the lanes of the same bin; by the whole warp
     auto drain = [&](bool out) {
-      const double ell = (static_cast<double>(ell_hi) + ell_lo) * ell_scale;
-      const double all = (power + (static_cast<double>(pw_hi) + pw_lo)) * p_norm;
+      const double ell = value(roots) * ell_scale, all = (power + value(squares)) * p_norm;
       unsigned left = __ballot_sync(0xffffffffu, out && count > 0 && bin >= 0 && bin < nbins);
       while (left) {
         const int leader = __ffs(left) - 1;
@@ -752,7 +786,7 @@ __global__ void __launch_bounds__(256) power_bin_kernel(const float2* __restrict
       }
       if (out) {
         power = 0.0;
-        pw_hi = pw_lo = ell_hi = ell_lo = 0.f;
+        squares = roots = Sum3{0.f, 0.f, 0.f};
         count = 0;
       }
     };
@@ -774,11 +808,11 @@ __global__ void __launch_bounds__(256) power_bin_kernel(const float2* __restrict
         const int each = iz == 0 || iz == m / 2 ? 1 : 2, modes = two ? 2 * each : each;
         const float scale = static_cast<float>(each);
         if (plain) {
-          add_square(u[i].x, scale, pw_hi, pw_lo);
-          add_square(u[i].y, scale, pw_hi, pw_lo);
+          add_square(squares, u[i].x, scale);
+          add_square(squares, u[i].y, scale);
           if (two) {
-            add_square(v[i].x, scale, pw_hi, pw_lo);
-            add_square(v[i].y, scale, pw_hi, pw_lo);
+            add_square(squares, v[i].x, scale);
+            add_square(squares, v[i].y, scale);
           }
         } else {
           double pw = static_cast<double>(u[i].x) * u[i].x + static_cast<double>(u[i].y) * u[i].y;
@@ -786,12 +820,7 @@ __global__ void __launch_bounds__(256) power_bin_kernel(const float2* __restrict
           power += each == 2 ? 2.0 * pw : pw;
         }
         count += modes;
-        // modes |n| as hi + lo, added with the rounding error kept (modes is a power of two)
-        const float a = static_cast<float>(n2), rest = static_cast<float>(n2 - static_cast<int>(a));
-        const float s = sqrtf(a), corr = (__fmaf_rn(-s, s, a) + rest) / (2.f * s);
-        const float x = s * modes, sum = ell_hi + x, back = sum - ell_hi;
-        ell_lo += ((ell_hi - (sum - back)) + (x - back)) + corr * modes;
-        ell_hi = sum;
+        add_root(roots, n2, modes);
       }
       __syncwarp();
     }
