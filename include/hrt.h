@@ -171,11 +171,12 @@ hrt_status hrt_pm_destroy(hrt_pm* pm); /* NULL is fine; synchronises the stream 
  * k-space kernel.  Returns HRT_ERR_CUDA if cuFFT refuses the callback. */
 hrt_status hrt_pm_set_fused(hrt_pm* pm, int32_t on);
 
-/* Split path of hrt_pm_solve (on by default for n = 256, 512, 1024): the library's own FFT passes along z, y and x,
- * with the k-space step of hrt_kspace_gradient inside the x pass, and back along y and z, so that every spectrum
- * crosses memory once per axis and no 3D spectrum is formed.  Same results as the 3D path (FP32 rounding of a
- * different FFT order).  on = 0 returns to 3D cuFFT plans and the separate k-space kernel.  HRT_ERR_INVALID_ARG for
- * other mesh sides. */
+/* Split path of hrt_pm_solve and, without ray fields, of hrt_pm_solve_adjoint (on by default for n = 64, 96, 128, 192,
+ * 256, 384, 512, 768 and 1024): the library's own FFT passes along z, y and x, with the k-space step of
+ * hrt_kspace_gradient inside the x pass, and back along y and z, so that every spectrum crosses memory once per axis
+ * and no 3D spectrum is formed.  Same results as the 3D path (FP32 rounding of a different FFT order).  on = 0
+ * returns to 3D cuFFT plans and the separate k-space kernel, on = 1 back to the passes: HRT_ERR_INVALID_ARG for
+ * other mesh sides, which have the 3D path only. */
 hrt_status hrt_pm_set_split(hrt_pm* pm, int32_t on);
 
 /* grad[3][n^3] <- gradient of phi from rho[n^3] (rho is overwritten as FFT scratch);
@@ -464,8 +465,9 @@ hrt_status hrt_mlp_to_bf16(const float* w_f32, void* w_bf16, void* stream);
 hrt_status hrt_kspace_table_adjoint(const void* gbar_hat, int32_t n_comp, const void* rho_hat, int64_t n, double box,
                                     double pref, const hrt_filter* f, float* table_bar, void* stream);
 
-/* Copies the density half spectrum of the last hrt_pm_solve into out (complex64 [n][n][n/2+1]); HRT_ERR_STATE
- * if that solve took the split path (see hrt_pm_set_split), which never forms the 3D spectrum. */
+/* The density half spectrum of the last hrt_pm_solve into out (complex64 [n][n][n/2+1]); not after a transposed solve on the
+ * object.  After a solve on the split path (see hrt_pm_set_split), which never forms the 3D spectrum, it is made on
+ * this request for n = 64, 96, 128, 192, 384 and 768, and HRT_ERR_STATE for n = 256, 512 and 1024. */
 hrt_status hrt_pm_density_spectrum(hrt_pm* pm, void* out);
 
 /* fields[n_out][n^3] <- gradient fields from a stored density half spectrum rho_hat (not modified): the k-space

@@ -327,7 +327,8 @@ namespace hrt {
 static size_t spectrum_bytes(int64_t n) { return static_cast<size_t>(n) * n * (n / 2 + 1) * sizeof(float2); }
 // Bytes of one spectrum buffer: the half spectrum, or the padded layout of the FFT passes where they exist.
 static size_t spectrum_alloc(int64_t n) { return fft_supported(n) ? fft_spectrum_bytes(n) : spectrum_bytes(n); }
-// Sides whose path the caller chooses (hrt_pm_set_split) and where a split solve leaves no spectrum to copy out.
+// Sides where a split solve leaves no spectrum to copy out: at the others, which took the 3D path before the passes had
+// their sides, hrt_pm_density_spectrum always answered.
 static bool split_side(int64_t n) { return n == 256 || n == 512 || n == 1024; }
 // Spectra the FFT passes need beyond the 4 (6 with ray fields) of the 3D path: the transformed density, two spectra
 // per filter set out of the x-pass and the fields between the inverse passes, the first of them in place of the
@@ -1108,7 +1109,8 @@ hrt_status hrt_pm_set_fused(hrt_pm* pm, int32_t on) {
 
 hrt_status hrt_pm_set_split(hrt_pm* pm, int32_t on) {
   if (!pm) return fail(HRT_ERR_INVALID_ARG, "pm is NULL");
-  if (on && !split_side(pm->n)) return fail(HRT_ERR_INVALID_ARG, "the split path needs a mesh side of 256, 512 or 1024");
+  if (on && !fft_supported(pm->n))
+    return fail(HRT_ERR_INVALID_ARG, "the split path needs a mesh side of 64, 96, 128, 192, 256, 384, 512, 768 or 1024");
   pm->split = on != 0;
   return HRT_OK;
 }
