@@ -39,7 +39,7 @@ typedef enum hrt_status {
   HRT_ERR_CUDA = 3,        /* a CUDA runtime or cuFFT call failed                                     */
   HRT_ERR_STATE = 4,       /* calls out of order (e.g. a step before particles exist), or poisoned    */
   HRT_ERR_NONFINITE = 5,   /* a NaN or infinity was found in an output that the call checks          */
-  HRT_ERR_TIMEOUT = 6      /* a host wait for the stream exceeded its limit                           */
+  HRT_ERR_TIMEOUT = 6      /* a host wait for the stream, or a kernel's for its copies, exceeded its limit */
 } hrt_status;
 
 /* Human-readable name of a status code (static string). */
@@ -180,9 +180,16 @@ hrt_status hrt_pm_set_fused(hrt_pm* pm, int32_t on);
 hrt_status hrt_pm_set_split(hrt_pm* pm, int32_t on);
 
 /* grad[3][n^3] <- gradient of phi from rho[n^3] (rho is overwritten as FFT scratch);
- * ray_grad[2][n^3] (only if the object has ray fields; else pass NULL) with the ray filter. */
+ * ray_grad[2][n^3] (only if the object has ray fields; else pass NULL) with the ray filter.  Asynchronous, as
+ * hrt_pm_solve_adjoint: should a kernel of the FFT passes give up waiting for its own copies (after about a second),
+ * its results are not sound; hrt_pm_status says so, and so does the next hrt_pm_solve, hrt_pm_solve_adjoint or
+ * hrt_pm_density_spectrum of the object that is called once it has happened, in place of its own work. */
 hrt_status hrt_pm_solve(hrt_pm* pm, float* rho, double pref, const hrt_filter* f, float* grad,
                         const hrt_filter* f_ray, float* ray_grad);
+
+/* Waits for the object's stream (within the host wait limit) and returns HRT_ERR_TIMEOUT if a kernel of a solve since
+ * the last report gave up waiting for its copies; the object stays usable. */
+hrt_status hrt_pm_status(hrt_pm* pm);
 
 /* ------------------------------------------------------------------------------------------------------
  * Rays
@@ -710,8 +717,12 @@ hrt_status hrt_read_wait(hrt_ctx* ctx);
  * particles, or no rays), and hrt_step / hrt_step_accumulate scan the particle state, the ray state and the
  * maps after the step and return HRT_ERR_NONFINITE if any value is not finite.  Each check waits for the
  * context's stream (within the host wait limit), so it costs a synchronisation and a pass over the state.
- * A kernel that gave up waiting for its own copies is reported here as HRT_ERR_TIMEOUT.  Neither status
- * poisons the context. */
+ * A tiled deposit that gave up waiting for its own copies (its results are sound) is reported here as
+ * HRT_ERR_TIMEOUT.  Neither status poisons the context.
+ * Without the checks too: should an FFT pass of the context's force give up waiting for its copies, the first call
+ * on the context after it has happened (hrt_read_wait, hrt_save_state, hrt_ctx_kappa_power and hrt_adjoint: also at
+ * their end) returns HRT_ERR_TIMEOUT, once and in place of its own work; the force is then gone (HRT_ERR_STATE) until
+ * particles are given or made again. */
 hrt_status hrt_set_nonfinite_check(hrt_ctx* ctx, int32_t on);
 
 /* Poisson prefactor of a static lens of total mass `mass` (Msun/h) in a periodic box of side `box` (Mpc/h):
@@ -732,8 +743,12 @@ hrt_status hrt_set_ray_theta_bits(hrt_ctx* ctx, int32_t bits);
  * variable HRT_FAIL_ALLOC_AT=k does the same from process start.  Process-wide; HRT_ERR_INVALID_ARG for k < 0. */
 hrt_status hrt_inject_alloc_failure(int64_t k);
 
+/* The same for a kernel's wait for its copies: the k-th hrt_pm_solve or hrt_pm_solve_adjoint on the FFT passes from now
+ * (those of contexts included) is marked as one that gave up waiting; k = 0 turns it off.  HRT_ERR_INVALID_ARG for k < 0. */
+hrt_status hrt_inject_wait_timeout(int64_t k);
+
 /* Process-wide limit, in seconds, of the library's host waits for a stream (hrt_kappa_power and
- * hrt_ctx_kappa_power waiting for the work already queued, the checks above); seconds <= 0 removes it (the
+ * hrt_ctx_kappa_power waiting for the work already queued, hrt_pm_status, the checks above); seconds <= 0 removes it (the
  * default).  When a wait exceeds it the call returns HRT_ERR_TIMEOUT; the queued work keeps running and the
  * call may be repeated.  HRT_ERR_INVALID_ARG for NaN. */
 hrt_status hrt_set_host_wait_limit(double seconds);

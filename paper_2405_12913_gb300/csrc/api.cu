@@ -80,6 +80,11 @@ bool inject_alloc_failure() {
   return g_alloc_count.fetch_add(1) + 1 == target;
 }
 
+// Host-side injection of a timed-out wait: the target-th solve on the FFT passes from the last reset (0: off).
+static std::atomic<long> g_timeout_left{0};
+
+static bool inject_wait_timeout() { return g_timeout_left.load() > 0 && g_timeout_left.fetch_sub(1) == 1; }
+
 hrt_status device_alloc(void** p, size_t bytes, cudaStream_t stream, const char* what) {
   *p = nullptr;
   if (bytes == 0) return HRT_OK;
@@ -318,7 +323,9 @@ struct hrt_pm {
   hrt::FftPlan fft;
   float2* twiddles = nullptr;
   void* split_hat = nullptr;  // work, until the callback plans need a larger one
-  int* xerr = nullptr;      // device error word of the kernels that wait for TMA copies (FFT passes, tiled deposit)
+  // Error word of the kernels that wait for TMA copies (FFT passes, tiled deposit), in pinned host memory: they write it
+  // only when a wait has timed out, and the host reads it without a copy or a wait.
+  int* xerr = nullptr;
   bool last_split = false;  // the last solve took the split path: rho_hat holds no 3D spectrum
 };
 
@@ -376,8 +383,9 @@ static hrt_status pm_make_split(hrt_pm* pm) {
   pm->split_hat = pm->work;
   std::vector<float2> tw;
   fft_twiddles(pm->n, tw);
-  HRT_TRY(device_alloc(reinterpret_cast<void**>(&pm->xerr), sizeof(int), pm->stream, "FFT pass error word"));
-  HRT_CUDA(cudaMemsetAsync(pm->xerr, 0, sizeof(int), pm->stream));
+  HRT_TRY(cuda_status(cudaHostAlloc(reinterpret_cast<void**>(&pm->xerr), sizeof(int), cudaHostAllocMapped | cudaHostAllocPortable),
+                      "FFT pass error word"));
+  *pm->xerr = 0;
   HRT_TRY(device_alloc(reinterpret_cast<void**>(&pm->twiddles), tw.size() * sizeof(float2), pm->stream, "twiddles"));
   HRT_CUDA(cudaMemcpyAsync(pm->twiddles, tw.data(), tw.size() * sizeof(float2), cudaMemcpyHostToDevice, pm->stream));
   // the host vector must outlive the copy
@@ -480,7 +488,7 @@ static void pm_release(hrt_pm* pm) {
   if (pm->have_cb2) cufftDestroy(pm->c2r_cb2);
   device_free(pm->twiddles, pm->stream);
   if (pm->split_hat != pm->work) device_free(pm->split_hat, pm->stream);
-  device_free(pm->xerr, pm->stream);
+  if (pm->xerr) cudaFreeHost(pm->xerr);
   device_free(pm->work, pm->stream);
   device_free(pm->rho_hat, pm->stream);
   device_free(pm->grad_hat, pm->stream);
@@ -527,6 +535,14 @@ static KspaceCallbackInfo callback_info(const hrt_pm* pm, const float* tab, cons
   return ci;
 }
 
+// HRT_ERR_TIMEOUT, once, if a kernel that has run since the last report gave up waiting for a tile's copy and set one of
+// `bits` (which are cleared).
+static hrt_status pm_timeouts(hrt_pm* pm, int bits, const char* what) {
+  if (!pm || !pm->xerr || !(__atomic_load_n(pm->xerr, __ATOMIC_ACQUIRE) & bits)) return HRT_OK;
+  __atomic_fetch_and(pm->xerr, ~bits, __ATOMIC_ACQ_REL);
+  return fail(HRT_ERR_TIMEOUT, "%s: a kernel gave up waiting for a tile's copy; what it wrote is not sound", what);
+}
+
 static FftSet fft_set(const hrt_pm* pm, const float* tab, const hrt_filter& f) {
   return FftSet{tab, tab + pm->n, f.g_table, f.g_nk, f.g_table ? static_cast<float>((f.g_nk - 1) / f.g_kmax) : 0.f};
 }
@@ -560,7 +576,9 @@ static hrt_status pm_solve(hrt_pm* pm, float* rho, double pref, const hrt_filter
     PhaseScope ps(pc, 5);
     HRT_TRY(launch_fft_inverse_y(pm->fft, pm->box, rays, pm->stream));
     if (before_fields) HRT_CUDA(cudaStreamWaitEvent(pm->stream, before_fields, 0));
-    return launch_fft_inverse_z(pm->fft, grad, rays ? ray_grad : nullptr, pm->stream);
+    HRT_TRY(launch_fft_inverse_z(pm->fft, grad, rays ? ray_grad : nullptr, pm->stream));
+    if (inject_wait_timeout()) __atomic_fetch_or(pm->xerr, kFftTimeout, __ATOMIC_RELAXED);
+    return HRT_OK;
   }
   {
     PhaseScope ps(pc, 3);
@@ -603,10 +621,18 @@ static hrt_status pm_solve(hrt_pm* pm, float* rho, double pref, const hrt_filter
 
 namespace hrt {
 
+// A timed-out wait in an FFT pass of the context's force, as far as the queued work has run: reported once, and the force
+// and what has been moved with it are gone (HRT_ERR_STATE until there are particles again).
+static hrt_status ctx_timeouts(hrt_ctx* ctx, const char* what) {
+  const hrt_status s = pm_timeouts(ctx->pm, kFftTimeout, what);
+  if (s != HRT_OK) ctx->force_valid = false;
+  return s;
+}
+
 static hrt_status ctx_guard(hrt_ctx* ctx) {
   if (!ctx) return fail(HRT_ERR_INVALID_ARG, "context is NULL");
   if (ctx->poisoned) return fail(HRT_ERR_STATE, "context is poisoned by an earlier CUDA error");
-  return HRT_OK;
+  return ctx_timeouts(ctx, "the force of an earlier call");
 }
 
 static hrt_status ctx_mark(hrt_ctx* ctx, hrt_status s) {
@@ -616,7 +642,7 @@ static hrt_status ctx_mark(hrt_ctx* ctx, hrt_status s) {
 
 // The opt-in check for NaN and infinity: scans the given arrays on the context's stream (after everything queued
 // so far), waits within the host wait limit and returns HRT_ERR_NONFINITE if any value is not finite.  Also
-// reports a kernel that gave up waiting for its own copies (the FFT passes' error word) as HRT_ERR_TIMEOUT.
+// reports a kernel that gave up waiting for its own copies (FFT passes, tiled deposit) as HRT_ERR_TIMEOUT.
 struct ScanItem {
   const void* p;
   int64_t n;
@@ -633,10 +659,10 @@ static hrt_status ctx_scan(hrt_ctx* ctx, std::initializer_list<ScanItem> items, 
     else HRT_TRY(launch_nonfinite_scan(static_cast<const float*>(it.p), it.n, ctx->finite_flag, st));
   }
   HRT_TRY(wait_stream(st, what));
-  int flag = 0, xerr = 0;
+  int flag = 0;
   HRT_CUDA(cudaMemcpy(&flag, ctx->finite_flag, sizeof(int), cudaMemcpyDeviceToHost));
-  if (ctx->pm && ctx->pm->xerr) HRT_CUDA(cudaMemcpy(&xerr, ctx->pm->xerr, sizeof(int), cudaMemcpyDeviceToHost));
-  if (xerr) return fail(HRT_ERR_TIMEOUT, "%s: a kernel gave up waiting for a tile's copy", what);
+  HRT_TRY(ctx_timeouts(ctx, what));
+  HRT_TRY(pm_timeouts(ctx->pm, kTileTimeout, what));
   if (flag) return fail(HRT_ERR_NONFINITE, "%s: a NaN or an infinity was found", what);
   return HRT_OK;
 }
@@ -1115,9 +1141,16 @@ hrt_status hrt_pm_set_split(hrt_pm* pm, int32_t on) {
   return HRT_OK;
 }
 
+hrt_status hrt_pm_status(hrt_pm* pm) {
+  if (!pm) return fail(HRT_ERR_INVALID_ARG, "pm is NULL");
+  HRT_TRY(wait_stream(pm->stream, "hrt_pm_status"));
+  return pm_timeouts(pm, kFftTimeout, "an earlier solve");
+}
+
 hrt_status hrt_pm_solve(hrt_pm* pm, float* rho, double pref, const hrt_filter* f, float* grad,
                         const hrt_filter* f_ray, float* ray_grad) {
   if (!pm || !rho || !grad) return fail(HRT_ERR_INVALID_ARG, "NULL argument");
+  HRT_TRY(pm_timeouts(pm, kFftTimeout, "an earlier solve"));
   if (ray_grad && pm->n_ray == 0) return fail(HRT_ERR_INVALID_ARG, "PM object has no ray fields");
   return pm_solve(pm, rho, pref, f, grad, f_ray, ray_grad);
 }
@@ -1326,14 +1359,18 @@ hrt_status hrt_particle_kick_drift_adjoint(const float* grad, int64_t n, double 
 hrt_status hrt_pm_solve_adjoint(hrt_pm* pm, float* grad_bar, double pref, const hrt_filter* f, float* ray_grad_bar,
                                 const hrt_filter* f_ray, float* rho_bar) {
   if (!pm || !grad_bar || !rho_bar) return fail(HRT_ERR_INVALID_ARG, "NULL argument");
+  HRT_TRY(pm_timeouts(pm, kFftTimeout, "an earlier solve"));
   HRT_TRY(check_filter(f));
   if (ray_grad_bar && (pm->n_ray == 0 || !f_ray)) return fail(HRT_ERR_INVALID_ARG, "PM object has no ray fields");
   if (ray_grad_bar) HRT_TRY(check_filter(f_ray));
   HRT_TRY(pm_tables(pm, *f, &pm->tab_a, &pm->key_a));
   if (ray_grad_bar) HRT_TRY(pm_tables(pm, *f_ray, &pm->tab_b, &pm->key_b));
   // fields of one filter set where the FFT passes run; with ray fields the 3D plans
-  if (pm->split && !ray_grad_bar)
-    return launch_fft_adjoint(pm->fft, pm->box, pref, fft_set(pm, pm->tab_a, *f), grad_bar, rho_bar, pm->stream);
+  if (pm->split && !ray_grad_bar) {
+    HRT_TRY(launch_fft_adjoint(pm->fft, pm->box, pref, fft_set(pm, pm->tab_a, *f), grad_bar, rho_bar, pm->stream));
+    if (inject_wait_timeout()) __atomic_fetch_or(pm->xerr, kFftTimeout, __ATOMIC_RELAXED);
+    return HRT_OK;
+  }
   const size_t sb = spectrum_bytes(pm->n), mb = static_cast<size_t>(pm->n) * pm->n * pm->n;
   char* gh = static_cast<char*>(pm->grad_hat);
   for (int j = 0; j < 3; ++j)
@@ -1694,6 +1731,7 @@ hrt_status hrt_pm_forward_fft(hrt_pm* pm, const float* real, void* out) {
 
 hrt_status hrt_pm_density_spectrum(hrt_pm* pm, void* out) {
   if (!pm || !out) return fail(HRT_ERR_INVALID_ARG, "NULL argument");
+  HRT_TRY(pm_timeouts(pm, kFftTimeout, "an earlier solve"));
   if (pm->last_split && !split_side(pm->n)) return launch_fft_spectrum(pm->fft, out, pm->stream);
   if (pm->last_split)
     return fail(HRT_ERR_STATE, "the last solve took the split path, which keeps no 3D spectrum (hrt_pm_set_split 0)");
@@ -2171,7 +2209,7 @@ hrt_status hrt_read_wait(hrt_ctx* ctx) {
   if (!ctx->copy_stream) return HRT_OK;
   HRT_TRY(ctx_mark(ctx, wait_stream(ctx->copy_stream, "hrt_read_wait")));
   ctx->copy_pending[0] = ctx->copy_pending[1] = false;
-  return HRT_OK;
+  return ctx_timeouts(ctx, "hrt_read_wait");
 }
 
 hrt_status hrt_read_particles(hrt_ctx* ctx, float* disp, float* mom, double* a_host, double* a_mom_host) {
@@ -2250,6 +2288,7 @@ hrt_status hrt_adjoint(hrt_ctx* ctx, const float* kappa_bar, const double* theta
   if (ctx->ray_stream) cudaStreamSynchronize(ctx->ray_stream);
   hrt_status s = tape_adjoint(ctx, kappa_bar, theta_bar, noise_bar, omega_bar_host);
   if (s == HRT_OK) s = cuda_status(cudaStreamSynchronize(ctx->stream), "adjoint sync");
+  if (s == HRT_OK) s = ctx_timeouts(ctx, "hrt_adjoint");
   return ctx_mark(ctx, s);
 }
 
@@ -2343,6 +2382,7 @@ hrt_status hrt_save_state(hrt_ctx* ctx, void* buf, size_t bytes) {
   if (ctx->maps) put(ctx->maps, 4 * r * static_cast<size_t>(ctx->cfg.n_sources) * sizeof(float));
   // the header copy reads host memory on the stream: wait before it goes out of scope
   if (s == HRT_OK) s = cuda_status(cudaStreamSynchronize(st), "save state");
+  if (s == HRT_OK) s = ctx_timeouts(ctx, "hrt_save_state");
   return ctx_mark(ctx, s);
 }
 
@@ -2395,7 +2435,8 @@ hrt_status hrt_ctx_kappa_power(hrt_ctx* ctx, int32_t source, int64_t m, double d
   if (!ctx->maps || source < 0 || source >= ctx->cfg.n_sources) return fail(HRT_ERR_INVALID_ARG, "no such map");
   if (m * m != ctx->rays.n_rays) return fail(HRT_ERR_INVALID_ARG, "rays do not form an m x m image");
   const float* kappa = ctx->maps + static_cast<int64_t>(source) * 4 * ctx->rays.n_rays;
-  return ctx_mark(ctx, hrt_kappa_power(kappa, m, dtheta, nbins, ell_min, ell_max, ell_host, p_host, count_host, ctx->stream));
+  HRT_TRY(ctx_mark(ctx, hrt_kappa_power(kappa, m, dtheta, nbins, ell_min, ell_max, ell_host, p_host, count_host, ctx->stream)));
+  return ctx_timeouts(ctx, "hrt_ctx_kappa_power");
 }
 
 hrt_status hrt_set_nonfinite_check(hrt_ctx* ctx, int32_t on) {
@@ -2426,6 +2467,12 @@ hrt_status hrt_set_ray_theta_bits(hrt_ctx* ctx, int32_t bits) {
 hrt_status hrt_inject_alloc_failure(int64_t k) {
   if (k < 0) return fail(HRT_ERR_INVALID_ARG, "k must be >= 0");
   set_alloc_failure(k);
+  return HRT_OK;
+}
+
+hrt_status hrt_inject_wait_timeout(int64_t k) {
+  if (k < 0) return fail(HRT_ERR_INVALID_ARG, "k must be >= 0");
+  g_timeout_left.store(static_cast<long>(k));
   return HRT_OK;
 }
 

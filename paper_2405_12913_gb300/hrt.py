@@ -79,6 +79,7 @@ _SIGS = {
     "hrt_kspace_gradient_noalloc": ([_P, _I64, _D, _D, _P, _I32, _P, _P, _I32, _P, _P], C.c_int),
     "hrt_pm_create": ([_I64, _D, _I32, _P, _P], C.c_int),
     "hrt_pm_destroy": ([_P], C.c_int),
+    "hrt_pm_status": ([_P], C.c_int),
     "hrt_pm_solve": ([_P, _P, _D, _P, _P, _P, _P], C.c_int),
     "hrt_pm_set_fused": ([_P, _I32], C.c_int),
     "hrt_pm_set_split": ([_P, _I32], C.c_int),
@@ -158,6 +159,7 @@ _SIGS = {
     "hrt_set_nonfinite_check": ([_P, _I32], C.c_int),
     "hrt_set_host_wait_limit": ([_D], C.c_int),
     "hrt_inject_alloc_failure": ([_I64], C.c_int),
+    "hrt_inject_wait_timeout": ([_I64], C.c_int),
     "hrt_set_ray_theta_bits": ([_P, _I32], C.c_int),
     "hrt_set_particle_correction": ([_P, _P], C.c_int),
     "hrt_static_prefactor": ([_D, _D, _P], C.c_int),
@@ -247,6 +249,11 @@ def hrt_static_prefactor(mass: float, box: float) -> float:
 def hrt_inject_alloc_failure(k: int):
     """Test hook: the k-th device allocation of the library from now reports out-of-memory (0: off)."""
     _check(_lib.hrt_inject_alloc_failure(k), "hrt_inject_alloc_failure")
+
+
+def hrt_inject_wait_timeout(k: int):
+    """Test hook: the k-th solve on the FFT passes from now is marked as one whose wait for a copy timed out (0: off)."""
+    _check(_lib.hrt_inject_wait_timeout(k), "hrt_inject_wait_timeout")
 
 
 def status_string(status: int) -> str:
@@ -367,6 +374,10 @@ class PM:
                                          _ptr(ray_grad_bar, torch.float32, "ray_grad_bar"),
                                          C.byref(f_ray) if f_ray is not None else None,
                                          _ptr(rho_bar, torch.float32, "rho_bar")), "hrt_pm_solve_adjoint")
+
+    def status(self):
+        """Waits for the solves so far; raises if a kernel of one gave up waiting for its copies."""
+        _check(_lib.hrt_pm_status(self._h), "hrt_pm_status")
 
     def density_spectrum(self, out: torch.Tensor):
         _check(_lib.hrt_pm_density_spectrum(self._h, _ptr(out, torch.complex64, "out")), "hrt_pm_density_spectrum")
