@@ -62,6 +62,25 @@ def test_sides_without_passes_have_nothing_to_report(hrt):
     pm.close()
 
 
+def test_objects_have_error_words_of_their_own(hrt):
+    # more objects than the library's page has words, some given back in between
+    f, rho = hrt.make_filter(4.0, 1.0), torch.ones(64, 64, 64, device="cuda")
+    grad = torch.empty(3, 64, 64, 64, device="cuda")
+    pms = [hrt.PM(64, 64.0) for _ in range(1030)]
+    for i in range(0, 1030, 2):
+        pms[i].close()
+    for i in range(0, 1030, 2):
+        pms[i] = hrt.PM(64, 64.0)
+    for i in (0, 1, 514, 1029):
+        hrt.hrt_inject_wait_timeout(1)
+        pms[i].solve(rho, 0.45, f, grad)
+    for i, pm in enumerate(pms):
+        if i in (0, 1, 514, 1029):
+            _raises(hrt, TIMEOUT, pm.status)
+        pm.status()
+        pm.close()
+
+
 def _context(hrt):
     ctx = hrt.Context(hrt.make_config(64, 64.0, 32, observer=(32.0, 32.0, 0.0), n_sources=1))
     g = torch.Generator(device="cuda").manual_seed(2)
