@@ -333,7 +333,8 @@ hrt_status hrt_raymesh_ray_step_tiled(hrt_raymesh* rm, const hrt_rays* rays, con
  * count per bin to host arrays of nbins.  kappa is m x m float32 (m even, 2 <= m <= 16384,
  * 1 <= nbins <= 256).  Synchronises the stream: it first waits for the work already queued on the stream
  * within the host wait limit (hrt_set_host_wait_limit) and returns HRT_ERR_TIMEOUT, having enqueued nothing,
- * when that expires; then its own transform and binning run and are waited for.
+ * when that expires; then its own transform and binning run and are waited for.  The plan and its buffers are kept for
+ * the next map of that side (hrt_release_workspaces).
  * ---------------------------------------------------------------------------------------------------- */
 hrt_status hrt_kappa_power(const float* kappa, int64_t m, double dtheta, int32_t nbins, double ell_min,
                            double ell_max, double* ell_host, double* p_host, int64_t* count_host,
@@ -511,8 +512,8 @@ hrt_status hrt_create(const hrt_config* cfg, void* stream, hrt_ctx** out);
 hrt_status hrt_destroy(hrt_ctx* ctx);  /* NULL is fine; synchronises the context's stream */
 
 /* Device bytes a context of this configuration allocates (plans and buffers, with the buffers of the default
- * particle sort), for capacity planning; the ray mesh, a recorded run for hrt_adjoint and up to 128 MB of workspace for
- * the planes of a ray step, which the library keeps between steps and gives back in hrt_destroy, come on top. */
+ * particle sort), for capacity planning; the ray mesh, a recorded run for hrt_adjoint and what the library keeps
+ * between calls (hrt_release_workspaces) come on top. */
 hrt_status hrt_workspace_bytes(const hrt_config* cfg, int64_t n_rays, size_t* bytes_host);
 
 /* Particles from Zel'dovich ICs (noise[n_side^3] device float32) at a_init, then the PM force at a_init. */
@@ -746,6 +747,13 @@ hrt_status hrt_inject_alloc_failure(int64_t k);
 /* The same for a kernel's wait for its copies: the k-th hrt_pm_solve or hrt_pm_solve_adjoint on the FFT passes from now
  * (those of contexts included) is marked as one that gave up waiting; k = 0 turns it off.  HRT_ERR_INVALID_ARG for k < 0. */
 hrt_status hrt_inject_wait_timeout(int64_t k);
+
+/* Device memory that the library keeps between calls, per device and whoever makes them (stateless calls and contexts):
+ * at most 256 MB of plans and spectra of hrt_kappa_power, and at most 128 MB of workspace of the planes that ray steps and
+ * ray-mesh kicks of many rays make; a captured call, or one that finds no memory for planes, goes without them.  This
+ * call gives back what is idle on the current device (so does hrt_destroy, and an allocation of the library that
+ * finds no memory before it is tried again); calls in other threads keep what they use. */
+hrt_status hrt_release_workspaces(void);
 
 /* Process-wide limit, in seconds, of the library's host waits for a stream (hrt_kappa_power and
  * hrt_ctx_kappa_power waiting for the work already queued, hrt_pm_status, the checks above); seconds <= 0 removes it (the

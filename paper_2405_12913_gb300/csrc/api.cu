@@ -89,7 +89,14 @@ hrt_status device_alloc(void** p, size_t bytes, cudaStream_t stream, const char*
   *p = nullptr;
   if (bytes == 0) return HRT_OK;
   if (inject_alloc_failure()) return fail(HRT_ERR_OOM, "%s: injected allocation failure", what);
-  return cuda_status(cudaMallocAsync(p, bytes, stream), what);
+  cudaError_t e = cudaMallocAsync(p, bytes, stream);
+  if (e == cudaErrorMemoryAllocation) {
+    // what the library keeps between calls may be what is missing
+    cudaGetLastError();
+    release_workspaces();
+    e = cudaMallocAsync(p, bytes, stream);
+  }
+  return cuda_status(e, what);
 }
 
 void device_free(void* p, cudaStream_t s) {
@@ -876,8 +883,8 @@ static hrt_status ctx_force(hrt_ctx* ctx) {
 // Plans and device buffers of the power spectrum, kept between calls: making the 2D plan and its buffers for a 2048^2
 // map took 1.3 ms of a 1.55 ms call.  A call takes an entry of its map side and device out of the pool (or makes one)
 // and gives it back once its stream is done with it, so that entries are never shared by threads or streams.  At most
-// kPowerPlans idle entries of at most kPowerPlanBytes together stay, the longest unused go first, and hrt_destroy
-// gives back all of its device's.
+// kPowerPlans idle entries of at most kPowerPlanBytes together stay, the longest unused go first, and hrt_destroy and
+// hrt_release_workspaces give back all of a device's.
 struct PowerPlan {
   int device = -1;
   int64_t m = 0;
@@ -904,7 +911,10 @@ static void power_plan_free(PowerPlan& w, cudaStream_t s) {
   device_free(w.spec, s);
   device_free(w.sums, s);
   cudaStreamSynchronize(s);
-  if (w.have_plan) cufftDestroy(w.plan);
+  if (w.have_plan) {
+    cufftSetStream(w.plan, nullptr);  // the stream of its last call may be gone
+    cufftDestroy(w.plan);
+  }
   w = PowerPlan{};
 }
 
@@ -923,7 +933,12 @@ static hrt_status power_plan_take(int64_t m, cudaStream_t s, PowerPlan& w) {
   w.m = m;
   const size_t spec = static_cast<size_t>(m) * (m / 2 + 1) * sizeof(float2);
   size_t work = 0;
-  hrt_status st = cufft_status(cufftPlan2d(&w.plan, static_cast<int>(m), static_cast<int>(m), CUFFT_R2C), "cufftPlan2d");
+  auto plan = [&] { return cufft_status(cufftPlan2d(&w.plan, static_cast<int>(m), static_cast<int>(m), CUFFT_R2C), "cufftPlan2d"); };
+  hrt_status st = plan();
+  if (st == HRT_ERR_OOM) {
+    release_workspaces();
+    st = plan();
+  }
   w.have_plan = st == HRT_OK;
   if (st == HRT_OK) st = cufft_status(cufftGetSize(w.plan, &work), "cufftGetSize");
   if (st == HRT_OK) st = device_alloc(&w.spec, spec, s, "kappa spectrum");
@@ -970,6 +985,12 @@ static void power_plans_release(int device, cudaStream_t s) {
     }
     power_plan_free(w, s);
   }
+}
+
+void release_workspaces() {
+  int device = 0;
+  if (cudaGetDevice(&device) == cudaSuccess) power_plans_release(device, cudaStreamPerThread);
+  ray_planes_release();
 }
 
 hrt_ray_geom ctx_geom(const hrt_config& c, const hrt_ctx* ctx) {
@@ -1815,9 +1836,7 @@ hrt_status hrt_destroy(hrt_ctx* ctx) {
       cudaEventDestroy(ev.second);
     }
   tape_free(ctx);
-  int device = 0;
-  if (cudaGetDevice(&device) == cudaSuccess) power_plans_release(device, s);
-  ray_planes_release();
+  release_workspaces();
   device_free(ctx->disp_alt, s);
   device_free(ctx->mom_alt, s);
   device_free(ctx->order_buf[0], s);
@@ -2496,6 +2515,11 @@ hrt_status hrt_set_ray_theta_bits(hrt_ctx* ctx, int32_t bits) {
 hrt_status hrt_inject_alloc_failure(int64_t k) {
   if (k < 0) return fail(HRT_ERR_INVALID_ARG, "k must be >= 0");
   set_alloc_failure(k);
+  return HRT_OK;
+}
+
+hrt_status hrt_release_workspaces(void) {
+  release_workspaces();
   return HRT_OK;
 }
 

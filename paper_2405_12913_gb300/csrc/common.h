@@ -24,7 +24,10 @@ bool inject_alloc_failure();
 // Resets the allocation count and makes the k-th device allocation from now fail (0: none); hrt_inject_alloc_failure.
 void set_alloc_failure(int64_t k);
 
-// cudaMallocAsync with the fault-injection hook; bytes == 0 gives nullptr.
+// Gives back the idle device memory that the library keeps between calls on the current device (hrt_release_workspaces).
+void release_workspaces();
+
+// cudaMallocAsync with the fault-injection hook, tried again after release_workspaces; bytes == 0 gives nullptr.
 hrt_status device_alloc(void** p, size_t bytes, cudaStream_t stream, const char* what);
 
 // Waits for the work queued on s, for at most the process-wide limit set by hrt_set_host_wait_limit (no limit

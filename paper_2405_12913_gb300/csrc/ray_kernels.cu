@@ -538,6 +538,7 @@ void* plane_workspace(size_t bytes, cudaStream_t s) {
     cudaGetLastError();
     return nullptr;
   }
+  if (inject_alloc_failure()) return nullptr;
   cudaMemPool_t pool = plane_pool();
   void* work = nullptr;
   if (pool && cudaMallocFromPoolAsync(&work, bytes, pool, s) == cudaSuccess) return work;

@@ -768,7 +768,13 @@ static hrt_status plan_for(hrt_raymesh* rm, int64_t n2d, cudaStream_t s, cufftHa
   auto it = rm->plans.find(n2d);
   if (it == rm->plans.end()) {
     cufftHandle h;
-    HRT_TRY(cufft_check(cufftPlan2d(&h, static_cast<int>(n2d), static_cast<int>(n2d), CUFFT_C2C), "plan"));
+    auto make = [&] { return cufft_check(cufftPlan2d(&h, static_cast<int>(n2d), static_cast<int>(n2d), CUFFT_C2C), "plan"); };
+    hrt_status st = make();
+    if (st == HRT_ERR_OOM) {  // as device_alloc
+      release_workspaces();
+      st = make();
+    }
+    HRT_TRY(st);
     it = rm->plans.emplace(n2d, h).first;
   }
   plan = it->second;

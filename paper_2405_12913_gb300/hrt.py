@@ -158,6 +158,7 @@ _SIGS = {
     "hrt_ctx_set_profiling": ([_P, _I32], C.c_int),
     "hrt_set_nonfinite_check": ([_P, _I32], C.c_int),
     "hrt_set_host_wait_limit": ([_D], C.c_int),
+    "hrt_release_workspaces": ([], C.c_int),
     "hrt_inject_alloc_failure": ([_I64], C.c_int),
     "hrt_inject_wait_timeout": ([_I64], C.c_int),
     "hrt_set_ray_theta_bits": ([_P, _I32], C.c_int),
@@ -244,6 +245,11 @@ def hrt_static_prefactor(mass: float, box: float) -> float:
     out = C.c_double()
     _check(_lib.hrt_static_prefactor(mass, box, C.byref(out)), "hrt_static_prefactor")
     return out.value
+
+
+def hrt_release_workspaces():
+    """Gives back the device memory that the library keeps idle between calls on the current device."""
+    _check(_lib.hrt_release_workspaces(), "hrt_release_workspaces")
 
 
 def hrt_inject_alloc_failure(k: int):
