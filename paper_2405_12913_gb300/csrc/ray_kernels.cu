@@ -574,7 +574,11 @@ hrt_status launch_ray_step(const hrt_rays& rays, const float* gx, const float* g
     }
   }
   if (work) {
-    HRT_CUDA(cudaMemsetAsync(work, 0, 256, s));
+    const cudaError_t cleared = cudaMemsetAsync(work, 0, 256, s);
+    if (cleared != cudaSuccess) {
+      cudaFreeAsync(work, s);
+      return cuda_status(cleared, "workspace of the ray planes");
+    }
     ray_bounds_kernel<<<std::min(blocks_for(rays.n_rays, 256), 152u * 8u), 256, 0, s>>>(
         reinterpret_cast<const ulonglong2*>(rays.theta), rays.n_rays, p, q);
     plane_kernel<<<152 * 8, 256, 0, s>>>(gx, gy, p, q);
