@@ -98,3 +98,63 @@ def test_planes_end_where_they_no_longer_pay(hrt, width, r, planes):
     _compare(whole, parts)
     # the planes' arithmetic is packed, so that of so many rays some round otherwise; the fields' is the parts'
     assert torch.equal(whole[1], parts[1]) != planes
+
+
+# mesh side, box, observer, half width of the bundle (rad), shell, spread of eta, samples per cell: a bundle within the box; one
+# wider than the box, off the origin; a shell towards the observer, with fewer samples than cells; rays that leave the
+# first half shell's cells in the second
+CASES = [(64, 100.0, (50.0, 50.0, 0.0), 0.02, (900.0, 1000.0), 0.0, 1.0),
+         (60, 60.0, (3.0, 61.0, 7.0), 0.05, (900.0, 950.0), 0.0, 1.0),
+         (96, 200.0, (100.0, 20.0, 0.0), 0.01, (700.0, 560.0), 0.0, 0.4),
+         (64, 100.0, (50.0, 50.0, 0.0), 0.005, (500.0, 700.0), 200.0, 2.0)]
+
+
+@pytest.mark.parametrize("case", range(len(CASES)))
+def test_bundles_that_reach_the_planes_match_the_fields(hrt, case):
+    n, box, obs, width, chi, spread, samples = CASES[case]
+    geom = hrt.make_geom(n, box, obs, samples)
+    nodes = sum(_nodes(hrt, geom, chi))
+    r = PLANE_WORK // nodes + 1
+    part = PLANE_WORK // nodes // 2
+    fields, theta = _bundle(n, r, width, case)
+    eta = spread * torch.randn(r, 2, device="cuda", generator=torch.Generator(device="cuda").manual_seed(case + 10))
+    whole = _step(hrt, fields, geom, theta, eta, chi, r)
+    parts = _step(hrt, fields, geom, theta, eta, chi, part)
+    _compare(whole, parts)
+    assert not torch.equal(whole[3], parts[3])  # the planes' packed arithmetic rounds some of so many rays otherwise
+    assert parts[3].abs().max() > 0
+
+
+@pytest.mark.parametrize("value", [float("inf"), float("nan"), 1e30])
+def test_an_angle_out_of_range_stays_its_own(hrt, value):
+    # in half shells of many nodes, of a bundle on the planes
+    n, chi, r = 64, (900.0, 1000.0), 70000
+    geom = hrt.make_geom(n, 100.0, (50.0, 50.0, 0.0))
+    assert r * sum(_nodes(hrt, geom, chi)) >= PLANE_WORK
+    fields, theta = _bundle(n, r, 0.01, 9)
+    eta = torch.zeros(r, 2, device="cuda")
+    want = _step(hrt, fields, geom, theta, eta, chi, r)
+    eta[7] = value  # its angle of the second half shell
+    got = _step(hrt, fields, geom, theta, eta, chi, r)
+    keep = torch.ones(r, dtype=torch.bool, device="cuda")
+    keep[7] = False
+    for a, b in zip(got, want):
+        assert torch.equal(a[keep], b[keep])
+    parts = _step(hrt, fields, geom, theta, eta, chi, r // 2)
+    assert not torch.equal(got[3][keep], parts[3][keep])  # the whole bundle's came from the planes
+
+
+def test_an_angle_that_is_not_finite_at_the_start_leaves_all_to_the_fields(hrt):
+    # the box of the rays is no sensible number of cells then
+    n, chi, r = 64, (900.0, 1000.0), 70000
+    geom = hrt.make_geom(n, 100.0, (50.0, 50.0, 0.0))
+    fields, theta = _bundle(n, r, 0.01, 9)
+    eta = torch.zeros(r, 2, device="cuda")
+    for value in (float("nan"), float("inf"), 1e12):
+        theta[5, 1] = value
+        whole = _step(hrt, fields, geom, theta, eta, chi, r)
+        parts = _step(hrt, fields, geom, theta, eta, chi, r // 2)
+        keep = torch.ones(r, dtype=torch.bool, device="cuda")
+        keep[5] = False
+        for a, b in zip(whole, parts):
+            assert torch.equal(a[keep], b[keep])
