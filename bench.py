@@ -259,49 +259,31 @@ def run_gpu(args, W, world, rank, local):
     disp0, mom0, _, _ = ctx.hrt_read_particles()
     grid = W.reverse_grid
     slots = {s: i for i, s in enumerate(W.source_steps)}
-    # own kernels per ray step: the direct gather is three launches (the rays' bounds, the node planes, the step; the last
-    # alone for a small bundle); the ray mesh is, per half shell, the copy of its planes, the projection and the filter
-    # (around cuFFT's transforms), then the ray kernel
-    ray_launches = 3 if W.n_rays >= 1 << 18 else 1
     if args.kick == "mesh":
         ctx.hrt_set_ray_mesh(raymesh_config(hrt, W))
-        ray_launches = 7 if W.n_rays >= 1 << 18 else 5
-
-    # own kernels per Poisson solve: the FFT passes along z, y, x and back, or the k-space kernel between cuFFT plans
-    solve_launches = 5 if own_fft(W) else 1
-    # the context sorts particles given by the caller before their first force, then every sort_every particle
-    # steps (6 own launches: cell keys, three scan passes, inversion, gather)
+    # the context sorts particles given by the caller before their first force, then every sort_every particle steps
     sort_every = 8 if args.sort_every is None else args.sort_every
-    since_sort = [0]
 
     def reset():
         ctx.hrt_init_particles(disp0, mom0, 1.0)
         ctx.hrt_init_rays(theta0)
-        since_sort[0] = 0
 
     reset.state = (disp0, mom0, theta0)
 
     def run_steps(k, start=0):
         """k reverse steps continuing at reverse index `start`, cycling through the reverse grid."""
-        launches = 0
         pos = start
         for _ in range(k):
             if pos == len(grid) - 1:
                 reset()
-                launches += 2 + solve_launches + (6 if sort_every > 0 else 0)  # sort, CIC scatter, solve, ray initialisation
                 pos = 0
             n = pos + 1
             ctx.hrt_step(grid[n], slots.get(n, -1))
-            launches += 1 + solve_launches + ray_launches  # kick-drift-deposit, Poisson solve, ray step
-            since_sort[0] += 1
-            if sort_every > 0 and since_sort[0] >= sort_every:
-                launches += 6
-                since_sort[0] = 0
             pos = n
-        return pos, launches
+        return pos
 
     reset()
-    pos, _ = run_steps(args.warmup)
+    run_steps(args.warmup)
     reset()  # the timed run starts at a = 1 like the workload
     pos = 0
     barrier()
@@ -309,9 +291,11 @@ def run_gpu(args, W, world, rank, local):
     clocks.start()
     t0 = torch.cuda.Event(enable_timing=True)
     t1 = torch.cuda.Event(enable_timing=True)
+    launches = hrt.hrt_kernel_launches()
     t0.record(stream)
-    pos, launches = run_steps(args.steps, pos)
+    pos = run_steps(args.steps, pos)
     t1.record(stream)
+    launches = hrt.hrt_kernel_launches() - launches  # the library's own, as it counts them
     barrier()
     clk = clocks.stop()
     ms_max = max_over_ranks(t0.elapsed_time(t1), world, dev)

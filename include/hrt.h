@@ -748,6 +748,9 @@ hrt_status hrt_inject_alloc_failure(int64_t k);
  * (those of contexts included) is marked as one that gave up waiting; k = 0 turns it off.  HRT_ERR_INVALID_ARG for k < 0. */
 hrt_status hrt_inject_wait_timeout(int64_t k);
 
+/* Kernels of the library (without cuFFT's) that this process has launched so far, captured ones included; host only. */
+hrt_status hrt_kernel_launches(int64_t* count_host);
+
 /* Device memory that the library keeps between calls, per device and whoever makes them (stateless calls and contexts):
  * at most 256 MB of plans and spectra of hrt_kappa_power, and at most 576 MB of workspace of the planes that ray steps and
  * ray-mesh kicks of many rays make; a captured call, or one that finds no memory for planes, goes without them.  This

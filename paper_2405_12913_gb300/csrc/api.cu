@@ -80,6 +80,8 @@ bool inject_alloc_failure() {
   return g_alloc_count.fetch_add(1) + 1 == target;
 }
 
+std::atomic<int64_t> g_kernel_launches{0};
+
 // Host-side injection of a timed-out wait: the target-th solve on the FFT passes from the last reset (0: off).
 static std::atomic<long> g_timeout_left{0};
 
@@ -2515,6 +2517,12 @@ hrt_status hrt_set_ray_theta_bits(hrt_ctx* ctx, int32_t bits) {
 hrt_status hrt_inject_alloc_failure(int64_t k) {
   if (k < 0) return fail(HRT_ERR_INVALID_ARG, "k must be >= 0");
   set_alloc_failure(k);
+  return HRT_OK;
+}
+
+hrt_status hrt_kernel_launches(int64_t* count) {
+  if (!count) return fail(HRT_ERR_INVALID_ARG, "count is NULL");
+  *count = g_kernel_launches.load();
   return HRT_OK;
 }
 

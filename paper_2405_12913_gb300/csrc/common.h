@@ -3,6 +3,7 @@
 
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cstdarg>
 #include <cstdint>
 #include <cstdio>
@@ -38,6 +39,10 @@ hrt_status wait_stream(cudaStream_t s, const char* what);
 hrt_status launch_nonfinite_scan(const float* p, int64_t n, int* flag, cudaStream_t s);
 hrt_status launch_nonfinite_scan(const double* p, int64_t n, int* flag, cudaStream_t s);
 
+// Kernels of the library launched by this process (hrt_kernel_launches).
+extern std::atomic<int64_t> g_kernel_launches;
+inline void count_launches(int n) { g_kernel_launches.fetch_add(n, std::memory_order_relaxed); }
+
 inline cudaStream_t as_stream(void* s) { return reinterpret_cast<cudaStream_t>(s); }
 
 inline unsigned blocks_for(int64_t n, int threads) {
@@ -55,4 +60,9 @@ inline unsigned blocks_for(int64_t n, int threads) {
 
 #define HRT_CUDA(expr) HRT_TRY(::hrt::cuda_status((expr), #expr))
 
-#define HRT_LAUNCHED(name) HRT_TRY(::hrt::cuda_status(cudaGetLastError(), name))
+// After one kernel launch.
+#define HRT_LAUNCHED(name)                                \
+  do {                                                    \
+    ::hrt::count_launches(1);                             \
+    HRT_TRY(::hrt::cuda_status(cudaGetLastError(), name)); \
+  } while (0)

@@ -598,6 +598,7 @@ hrt_status launch_ray_step(const hrt_rays& rays, const float* gx, const float* g
   kernel<<<blocks_for(rays.n_rays, 128), 128, work ? nodes * sizeof(float4) : 0, s>>>(
       reinterpret_cast<double2*>(rays.theta), reinterpret_cast<float2*>(rays.eta),
       reinterpret_cast<float4*>(rays.A), reinterpret_cast<float4*>(rays.B), rays.n_rays, gx, gy, p, maps, gz, q);
+  count_launches(work ? 3 : 1);
   const cudaError_t launched = cudaGetLastError();
   if (work) cudaFreeAsync(work, s);
   return cuda_status(launched, "ray_step_kernel");

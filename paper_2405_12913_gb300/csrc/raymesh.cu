@@ -847,6 +847,7 @@ static hrt_status project_planes(const float* gx, const float* gy, const Project
     raymesh_planes_kernel<<<tiles * chunks, 256, 0, s>>>(gx, gy, p, v);
     const dim3 grid(static_cast<unsigned>((p.n2d + kTileY - 1) / kTileY), static_cast<unsigned>(rows / kTileX));
     raymesh_project_narrow_kernel<<<grid, kTileX * kTileY, 0, s>>>(p, mesh, v);
+    count_launches(2);
     done = row + rows >= p.n2d;
   }
   const cudaError_t launched = cudaGetLastError();

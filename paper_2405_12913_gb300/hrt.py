@@ -158,6 +158,7 @@ _SIGS = {
     "hrt_ctx_set_profiling": ([_P, _I32], C.c_int),
     "hrt_set_nonfinite_check": ([_P, _I32], C.c_int),
     "hrt_set_host_wait_limit": ([_D], C.c_int),
+    "hrt_kernel_launches": ([_P], C.c_int),
     "hrt_release_workspaces": ([], C.c_int),
     "hrt_inject_alloc_failure": ([_I64], C.c_int),
     "hrt_inject_wait_timeout": ([_I64], C.c_int),
@@ -244,6 +245,13 @@ def hrt_static_prefactor(mass: float, box: float) -> float:
     """4 pi G M / box^3: the Poisson prefactor of a static lens of mass M (Msun/h) in a box of side L (Mpc/h)."""
     out = C.c_double()
     _check(_lib.hrt_static_prefactor(mass, box, C.byref(out)), "hrt_static_prefactor")
+    return out.value
+
+
+def hrt_kernel_launches() -> int:
+    """Kernels of the library (without cuFFT's) that this process has launched so far."""
+    out = C.c_int64()
+    _check(_lib.hrt_kernel_launches(C.byref(out)), "hrt_kernel_launches")
     return out.value
 
 
