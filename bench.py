@@ -29,11 +29,13 @@ sys.path.insert(0, ROOT)
 
 METRIC = "HRT sim-steps/s (512³ p,1024³ mesh,4M rays) vs plain path at κ P(ℓ) err<1%"
 UNIT = "sim-steps/s"
+# files that hold a phase's device code: its kernels and the headers with the device functions they use
 KERNEL_SOURCES = {
-    "ray_step": ["ray_kernels.cu", "mesh_kernels.h"],
+    "ray_step": ["ray_kernels.cu", "mesh_kernels.h", "packed.cuh", "ray_position.cuh", "readout.cuh"],
     "kick_drift": ["mesh_kernels.cu"],
     "cic_scatter": ["mesh_kernels.cu"],
-    "kspace": ["mesh_kernels.cu", "fft_passes.cu", "fft_passes.cuh", "tma.h"],
+    "kspace": ["mesh_kernels.cu", "fft_passes.cu", "fft_passes.cuh", "fft_passes.h", "fft_passes_mid.cu",
+               "fft_passes_small.cu", "packed.cuh", "tma.h"],
 }
 
 
