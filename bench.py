@@ -7,6 +7,9 @@ from 1 to 1/3 (source planes z = 0.5, 1, 2), synthetic Zel'dovich ICs evolved fo
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl gb300|reference]
 
+One JSON line with the result goes to standard output; on one GPU a second one with the tables of the widened rows, the
+precision and the learned forms goes to standard error.
+
 Under torchrun each rank runs an independent replica (its own seed); the timed region is bracketed by a
 barrier and a device synchronise, and rank 0 reports the maximum over ranks.  The reference arm times the
 FP64 CPU oracle on a bounded sample of the same workload.
@@ -746,6 +749,18 @@ def precision_errors():
     return out
 
 
+DETAILS = ("next_rows", "precision", "learned")
+
+
+def report(line):
+    """The result as one short JSON line on standard output, and before it the tables of the widened rows, the precision
+    and the learned forms (20 KB) as one on standard error."""
+    details = {k: line[k] for k in DETAILS if line.get(k) is not None}
+    if details:
+        print(json.dumps({"details_of": line["config"]["workload"], **details}), file=sys.stderr, flush=True)
+    print(json.dumps({k: v for k, v in line.items() if k not in DETAILS}))
+
+
 def main():
     args = parse()
     world, rank, local = dist_env()
@@ -771,7 +786,7 @@ def main():
                                 "measured_at_sample_size": {
                                     "value": 1.0 / t_sample, "unit": UNIT,
                                     "workload": f"{n_side}^3 particles, {n_mesh}^3 mesh, {n_pix}^2 rays (timed directly)"}}
-    print(json.dumps(line))
+    report(line)
     return 0
 
 
